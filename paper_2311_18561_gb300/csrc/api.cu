@@ -192,7 +192,7 @@ struct pvg_frame {
     DevBuf tile_order_bwd;      // [tiles] adjoint launch order (by walk)
     DevBuf pix_T, pix_last;     // [pixels]
     DevBuf pix_neval;           // [pixels]
-    DevBuf g2d;                 // [NV * 10] image-space gradients by depth position
+    DevBuf g2d;                 // [NV] image-space gradients by depth position (g2_bytes)
     DevBuf gfeat;               // [NV * F] dL/d(channel value)
     std::vector<ViewDesc> views;
     int feat_mask = 0, n_feat = 0, n_sem = 0;  // extra channels of the forward
@@ -637,6 +637,9 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
     p.vis_off = ptr<uint32_t>(x->vis_off);
     p.feat_mask = fmask;
     p.n_feat = n_feat;
+    if (!keep_state) p.pix_T = nullptr;  // inference only: no state for a backward pass
+    // with state: each tile's walk length, from which the adjoint orders its tiles
+    p.tile_walk = keep_state ? ptr<uint32_t>(f->tile_walk) : nullptr;
     StageTimer &tm = x->timer;
     const bool timer_on = tm.on;
     if (capturing) tm.on = false;
@@ -712,9 +715,6 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
     }
     f->pair_capacity = pair_cap;
     p.pair_vals = ptr<uint32_t>(f->pair_vals);
-    if (!keep_state) p.pix_T = nullptr;  // inference only: no state for a backward pass
-    // with state: each tile's walk length, from which the adjoint orders its tiles
-    p.tile_walk = keep_state ? ptr<uint32_t>(f->tile_walk) : nullptr;
     tm.begin(PVG_STAGE_COMPOSITE, s);
     launch_composite(p, s);
     if (n_feat) launch_composite_feat(p, s);
@@ -894,7 +894,7 @@ extern "C" pvg_status_t pvg_render_bwd(pvg_ctx_t *x, const pvg_scene_t *scene, c
     if ((f->feat_mask & kFeatSem) && grads->sem)
         PVG_CUDA(cudaMemsetAsync(grads->sem, 0, sizeof(float) * N * (size_t)f->n_sem, s));
     if (f->n_items == 0 && !scene->sky) return PVG_OK;
-    PVG_TRY(ensure_c(f->g2d, sizeof(float) * 10 * (size_t)f->n_items, capturing));
+    PVG_TRY(ensure_c(f->g2d, g2_bytes(f->n_items), capturing));
     if (feat_bwd) PVG_TRY(ensure_c(f->gfeat, sizeof(float) * f->n_feat * (size_t)f->n_items, capturing));
     PVG_TRY(stage_views(*f->stage_bwd, views, s, capturing));
 
@@ -922,7 +922,8 @@ extern "C" pvg_status_t pvg_render_bwd(pvg_ctx_t *x, const pvg_scene_t *scene, c
     p.tile_order = ptr<uint32_t>(f->tile_order);
     p.pix_T = ptr<float>(f->pix_T);
     p.pix_last = ptr<uint32_t>(f->pix_last);
-    p.g2d = ptr<float>(f->g2d);
+    p.g2m = ptr<double>(f->g2d);
+    p.g2d = reinterpret_cast<float *>(ptr<char>(f->g2d) + g2d_offset(f->n_items));
     for (const ViewDesc &d : views) p.aux |= (d.dl_depth || d.dl_alpha || d.sky) ? 1 : 0;
     if (feat_bwd) {
         p.feat_mask = f->feat_mask;

@@ -155,7 +155,6 @@ __global__ void __launch_bounds__(kFeatBlock) k_composite_feat_bwd(Params P) {
                     }
                     if (raw <= kAlphaCap) {
                         const float ga = Ti * X - inv * S[p];
-                        gv[5] += ga * G;
                         const float gpow = ga * alpha;
                         const float my = gpow * dy;
                         A0 += gpow;
@@ -169,6 +168,7 @@ __global__ void __launch_bounds__(kFeatBlock) k_composite_feat_bwd(Params P) {
                     gv[0] = dx * A0;
                     gv[2] = dx * gv[0];
                     gv[3] = dx * gv[1];
+                    gv[5] = A0;
                     constexpr int N0 = NT >= 32 ? 32 : pow2_at_least(NT);
                     reduce_chunk<NT, 0, N0>(gv, s_acc, k);
                     if constexpr (NT > 32) reduce_chunk<NT, 32, pow2_at_least(NT - 32)>(gv, s_acc, k);
@@ -183,17 +183,15 @@ __global__ void __launch_bounds__(kFeatBlock) k_composite_feat_bwd(Params P) {
             for (int k = tid; k < cnt; k += blockDim.x) {
                 const float *a = &s_acc[k * NT];
                 const float ap = s0[k].z, bp = s0[k].w, cp = s1[k].x;
-                float gt[6];
-                gt[0] = -0.6931471805599453f * (2.f * ap * a[0] + bp * a[1]);
-                gt[1] = -0.6931471805599453f * (bp * a[0] + 2.f * cp * a[1]);
-                gt[2] = -0.5f * a[2];
-                gt[3] = -a[3];
-                gt[4] = -0.5f * a[4];
-                gt[5] = a[5];
-                float *dst = &P.g2d[10 * (size_t)s_m[k]];
+                const size_t m = s_m[k];
+                const float gu = -0.6931471805599453f * (2.f * ap * a[0] + bp * a[1]);
+                const float gv = -0.6931471805599453f * (bp * a[0] + 2.f * cp * a[1]);
+                if (gu != 0.f) atomicAdd(P.g2d + kG2dRow * m, gu);
+                if (gv != 0.f) atomicAdd(P.g2d + kG2dRow * m + 1, gv);
+                if (a[5] != 0.f) atomicAdd(P.g2d + kG2dRow * m + kG2dPower, a[5]);
 #pragma unroll
-                for (int c = 0; c < 6; c++)
-                    if (gt[c] != 0.f) atomicAdd(dst + c, gt[c]);
+                for (int c = 0; c < 3; c++)
+                    if (a[2 + c] != 0.f) atomicAdd(P.g2m + 3 * m + c, (double)a[2 + c]);
                 float *gf = &P.gfeat[(size_t)s_m[k] * P.n_feat];
                 for (int c = 0; c < P.n_feat; c++)
                     if (a[6 + c] != 0.f) atomicAdd(gf + c, a[6 + c]);

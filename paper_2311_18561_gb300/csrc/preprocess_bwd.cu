@@ -122,9 +122,13 @@ __device__ __forceinline__ bool item_adjoint(const Params &P, const ViewDesc &V,
     constexpr int K = (D + 1) * (D + 1);
     Fwd F;
     if (!project(V, i, P.dilation, P.tile_w, P.tile_h, F)) return false;
-    const float *G2 = P.g2d + 10 * (size_t)m;
-    const float gu = G2[0], gv = G2[1], ga = G2[2], gb = G2[3], gc = G2[4];
-    const float got = G2[5], gz = G2[9];
+    const float4 *G2 = reinterpret_cast<const float4 *>(P.g2d + kG2dRow * (size_t)m);
+    const float4 g0 = G2[0], g1 = G2[1];  // u, v, power, r | g, b, z, -
+    const double *mom = P.g2m + 3 * (size_t)m;
+    // the moments as gradients of the conic (power = ln o~ - (a dx^2 + 2 b dx
+    // dy + c dy^2) / 2)
+    const float gu = g0.x, gv = g0.y, got = g0.z / F.ot, gz = g1.z;
+    const float ga = -0.5f * (float)mom[0], gb = -(float)mom[1], gc = -0.5f * (float)mom[2];
     float gmut[3] = {0.f, 0.f, 0.f};
     float gp[3] = {0.f, 0.f, 0.f};
     // ---- conic = inverse(cov2): dL/dcov2 = -Q Ghat Q
@@ -220,7 +224,7 @@ __device__ __forceinline__ bool item_adjoint(const Params &P, const ViewDesc &V,
     // two streaming passes over the coefficients (dL/dsh from Y, then
     // dL/ddir from dY) keep few values live at a time.
     {
-        const float gcol[3] = {G2[6], G2[7], G2[8]};
+        const float gcol[3] = {g0.w, g1.x, g1.y};
         float dx = F.mut.x - V.campos[0], dy = F.mut.y - V.campos[1], dz = F.mut.z - V.campos[2];
         const float dist = sqrtf(dx * dx + dy * dy + dz * dz);
         const float inv = 1.0f / dist;

@@ -82,7 +82,9 @@ struct Params {
     int32_t n_views;
     int32_t sh_degree;       // of the call's scene (kernels are specialised on it)
     int32_t tile_w, tile_h;
-    int32_t px;              // pixels per compositing thread
+    int32_t px;              // pixels per compositing thread of the configuration
+    int32_t block_shift;     // log2 of the width of a warp's pixel block (compositing kernels)
+    uint32_t blocks_per_tile;  // warps' pixel blocks in a tile
     float dilation;
     uint32_t n_items;        // NV
     uint32_t total_tiles;
@@ -116,14 +118,22 @@ struct Params {
     uint32_t *pix_last;      // [sum HW] list position after the last blend
     uint32_t *pix_neval;     // [2][sum HW] stats pass: in-footprint entries up to the stop, and blended ones
     // backward
-    float *g2d;              // [M*10] image-space gradients by depth position (u, v, conic a b c,
-                             // o~, colour with the forward's clamp applied, z)
+    double *g2m;             // [M*3] moments m_xx, m_xy, m_yy of dL/dpower over the pixels' offsets from
+                             // (u, v), by depth position
+    float *g2d;              // [M*kG2dRow] the other image-space gradients (rows of one 32-byte sector)
     int32_t aux;             // backward: some view has depth / opacity-map gradients or a sky map
     // extra channels
     int32_t feat_mask;       // kFeat* bits (0: none)
     int32_t n_feat;          // F
     float *gfeat;            // [M*F] dL/d(channel value) per visible item
 };
+
+// a row of g2d: u, v, the exponent (o~ dL/do~), the colour with the forward's
+// clamp applied, z
+constexpr int kG2dRow = 8, kG2dPower = 2, kG2dColour = 3, kG2dDepth = 6;
+// bytes of g2m and g2d for n items (g2m first, g2d at a 32-byte boundary)
+inline size_t g2d_offset(size_t n) { return (3 * sizeof(double) * n + 31) / 32 * 32; }
+inline size_t g2_bytes(size_t n) { return g2d_offset(n) + sizeof(float) * kG2dRow * n; }
 
 // view of a global item / tile by binary search over the per-view bases
 __device__ __forceinline__ int view_of_item(const ViewDesc *views, int nv, uint32_t gid) {
@@ -162,8 +172,8 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // tall), and a NaN coefficient stays NaN.
 constexpr float kMinRowCoef = 1e-20f;
 
-__device__ __forceinline__ void record_terms(const float4 *rec, uint32_t m, float4 &s0, float2 &s1, float4 &s2) {
-    const float4 a = rec[3 * (size_t)m], b = rec[3 * (size_t)m + 1], c = rec[3 * (size_t)m + 2];
+__device__ __forceinline__ void record_terms(const float4 *rec, size_t m, float4 &s0, float2 &s1, float4 &s2) {
+    const float4 a = rec[3 * m], b = rec[3 * m + 1], c = rec[3 * m + 2];
     s0 = make_float4(a.x, a.y, -0.5f * kLog2e * a.z, -kLog2e * a.w);
     const float cp = -0.5f * kLog2e * b.x;
     s1 = make_float2(cp > -kMinRowCoef ? -kMinRowCoef : cp, b.y);
@@ -477,8 +487,10 @@ void scan_count_pairs(const Params &p, void *temp, cudaStream_t s);
 void scan_emit_pairs(const Params &p, void *temp, cudaStream_t s);
 size_t emit_chunks(uint32_t capacity);
 void launch_ranges(const Params &p, cudaStream_t s);
+// the compositor's launch order; also zeroes p.tile_walk (if given), into
+// which the compositor's warps take maxima
 void launch_tile_order(const Params &p, cudaStream_t s);
-// the adjoint's first kernel: p.g2d rows of the visible items zeroed, and
+// the adjoint's first kernel: p.g2m and p.g2d rows of the visible items zeroed, and
 // the adjoint's tile order by walk[tile] (longest first) into order
 void launch_bwd_prep(const Params &p, const uint32_t *walk, uint32_t *order, cudaStream_t s);
 // raster

@@ -1,31 +1,40 @@
 // raster.cu -- per-tile compositing (stage c).
 //
 // Sec. 3.1, Eq. 3 with the depth and opacity channels Sec. 3.1 renders
-// beside colour: one CTA per tile of TW x TH pixels, TW x TH/PX threads, each
-// thread PX vertically adjacent pixels, each warp an 8 x 4 block of
-// threads.  The tile's sorted list is walked front to back in batches of
-// one record per thread, staged in shared memory as
-//   s0 = (u, v, a', b')   projected mean, conic pre-scaled by -log2(e)
-//   s1 = (c', o~)
-//   s2 = (r, g, b, z)
-// so a pixel's weight is one SFU ex2:
-//   alpha = min(0.99, o~ 2^(a' dx^2 + b' dx dy + c' dy^2)).
-// A pixel skips alpha < 1/255, stops before a blend that would leave
-// T < 1e-4, and accumulates C += c alpha T, D += z alpha T, O += alpha T;
-// the CTA leaves the list as soon as every pixel has stopped.  Several
-// pixels per thread share each shared-memory load and the loop overhead.
-// Every pixel's arithmetic is the same expression whatever TW, TH and PX,
-// so images are bit-identical across tile shapes.
-#include <type_traits>
+// beside colour: one warp per block of 32 PX pixels (raster_common.cuh),
+// which walks its tile's sorted list front to back.  A pixel's weight is one
+// SFU ex2,
+//   alpha = min(0.99, o~ 2^(a' dx^2 + b' dx dy + c' dy^2)),
+// with the conic pre-scaled by -log2(e).  A pixel skips alpha < 1/255, stops
+// before a blend that would leave T < 1e-4, and accumulates C += c alpha T,
+// D += z alpha T, O += alpha T.  Every pixel's arithmetic is the same
+// expression whatever the tile and block shapes, so images are bit-identical
+// across them.
+#include <climits>
 
 #include "raster_common.cuh"
 
 namespace pvg {
 namespace {
 
+// Entries whose alphas are evaluated together, before the chain of their
+// transmittances: a lone warp (the longest walk of a frame, the small
+// frames) waits on latencies, which four independent evaluations overlap
+// (two 641x479-sized views of 250k Gaussians: 350 us with 2, 280 us with 4).
+constexpr int kFwdUnroll = 4;
+// Resident warps per SM that the registers are held to, by pixels per lane:
+// without spills (16 warps of 128 registers against 20 of 96: 280 and 310 us
+// on those views, 193 and 195 us on the 1.5M-Gaussian 1920x1280 frame).
+constexpr int kFwdWarps4 = 16, kFwdWarps2 = 20;
+// Blocks of 128 pixels per SM from which a lane takes four pixels and not
+// two: below it the longest walk bounds the pass and two pixels per lane
+// shorten it (9,100 blocks: 186 us with two, 280 us with four); above it the
+// issue slots do (19,200 blocks: 243 and 193 us).
+constexpr int kFwdWide = 64;
+
 // Writes the images (and the saved per-pixel state) of a thread's PX pixels.
 template <int PX>
-__device__ __forceinline__ void composite_epilogue(const Params &P, const ViewDesc &V, const TileGeom &G,
+__device__ __forceinline__ void composite_epilogue(const Params &P, const ViewDesc &V, const BlockGeom &G,
                                                    const float (&T)[PX], const float (&C0)[PX],
                                                    const float (&C1)[PX], const float (&C2)[PX],
                                                    const float (&D)[PX], const float (&O)[PX],
@@ -64,265 +73,244 @@ __device__ __forceinline__ void composite_epilogue(const Params &P, const ViewDe
     }
 }
 
-// The tile's largest last-blend position (how far its adjoint walks),
-// by every thread of the CTA once its pixels are written.
+// The compositor: a warp walks its block's hits front to back, its pixels as
+// packed pairs of vertically adjacent ones (the falloff, alpha,
+// transmittance and accumulation of both take one .f32x2 instruction each).
+// A pixel that does not blend (alpha < 1/255, stopped, outside the image)
+// has its alpha zeroed: its weight is then 0 and its T and sums keep their
+// bits, so a warp takes no branch per pixel; entries with non-finite terms,
+// for which 0 weights would not do, take the one-pixel-at-a-time path.  The
+// sums are kept negated (the weight is -alpha T), which packed arithmetic
+// needs no negation for.
 template <int PX>
-__device__ __forceinline__ void tile_walk_record(const Params &P, const uint32_t (&last)[PX]) {
-    __shared__ uint32_t s_walk;
-    uint32_t m = last[0];
-#pragma unroll
-    for (int p = 1; p < PX; p++) m = max(m, last[p]);
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (threadIdx.x == 0) s_walk = 0u;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) atomicMax(&s_walk, m);
-    __syncthreads();
-    if (threadIdx.x == 0) P.tile_walk[P.tile_order ? P.tile_order[blockIdx.x] : blockIdx.x] = s_walk;
-}
-
-// kStats: instead of images, write per pixel the number of list entries
-// whose footprint box contains the pixel, up to and including the one
-// that stopped it (the compositing work E), and the number of those with
-// alpha >= 1/255 (blended, or stopping the pixel).
-template <int TW, int TH, int PX, bool kStats>
-__global__ void __launch_bounds__(TW *TH / PX) k_composite(Params P) {
-    pdl_enter();
-    constexpr int BLOCK = TW * TH / PX;
-    constexpr uint32_t ALL = (1u << PX) - 1u;
-    __shared__ float4 s0[BLOCK];
-    __shared__ float2 s1[BLOCK];
-    __shared__ float4 s2[BLOCK];
-    __shared__ float2 s_half[kStats ? BLOCK : 1];
-    const TileGeom G = tile_geom<TW, TH, PX>(P);
-    const ViewDesc &V = *G.V;
-    const uint2 r = G.r;
-    const int tid = threadIdx.x;
-    const float fx = (float)G.px + 0.5f;
-    float fy[PX];
-    float T[PX], C0[PX], C1[PX], C2[PX], D[PX], O[PX];
-    uint32_t last[PX], neval[PX], nblend[PX];
-    uint32_t done = 0;
-#pragma unroll
-    for (int p = 0; p < PX; p++) {
-        fy[p] = (float)(G.py0 + p) + 0.5f;
-        T[p] = 1.0f;
-        C0[p] = C1[p] = C2[p] = D[p] = O[p] = 0.f;
-        last[p] = 0;
-        neval[p] = 0;
-        nblend[p] = 0;
-        if (!(G.px < V.W && G.py0 + p < V.H)) done |= 1u << p;
-    }
-    for (uint32_t base = r.x; base < r.y; base += BLOCK) {
-        if (__syncthreads_count(done != ALL) == 0) break;
-        const uint32_t j = base + tid;
-        if (j < r.y) {
-            const uint32_t m = P.pair_vals[j];
-            stage_record(P, m, s0, s1, s2, tid);
-            if constexpr (kStats) s_half[tid] = make_float2(P.rec[3 * (size_t)m + 1].w, P.rec[3 * (size_t)m + 2].w);
-        }
-        __syncthreads();
-        const int cnt = (int)min((uint32_t)BLOCK, r.y - base);
-        for (int k = 0; k < cnt && done != ALL; k++) {
-            const float4 g = s0[k];
-            const float2 q = s1[k];
-            const float4 col = s2[k];
-            const uint32_t pos = base + k + 1 - r.x;  // list position after this entry
-            const float dx = __fsub_rn(fx, g.x);
-            const FalloffColumn fc = falloff_column(g.z, g.w, dx);
-            // entries whose o~ cannot reach the cap skip min(cap, .)
-            auto pixels = [&](auto capped) {
-                constexpr bool kCap = decltype(capped)::value;
-#pragma unroll
-                for (int p = 0; p < PX; p++) {
-                    if (done & (1u << p)) continue;
-                    const float dy = __fsub_rn(fy[p], g.y);
-                    if constexpr (kStats) {
-                        const float2 h = s_half[k];
-                        if (fabsf(dx) <= h.x && fabsf(dy) <= h.y) neval[p]++;
-                    }
-                    const float e = falloff_exp2(fc, q.x, dy);
-                    const float raw = __fmul_rn(q.y, ex2_approx(e));
-                    if (!(raw >= kAlphaMin)) continue;  // = min(cap, raw) < 1/255, cap > 1/255
-                    const float alpha = kCap ? fminf(kAlphaCap, raw) : raw;
-                    if constexpr (kStats) nblend[p]++;
-                    const float w = __fmul_rn(alpha, T[p]);
-                    const float Tn = __fsub_rn(T[p], w);
-                    if (Tn < kTStop) {
-                        done |= 1u << p;
-                        continue;
-                    }
-                    C0[p] = __fmaf_rn(col.x, w, C0[p]);
-                    C1[p] = __fmaf_rn(col.y, w, C1[p]);
-                    C2[p] = __fmaf_rn(col.z, w, C2[p]);
-                    D[p] = __fmaf_rn(col.w, w, D[p]);
-                    O[p] = __fadd_rn(O[p], w);
-                    T[p] = Tn;
-                    last[p] = pos;
-                }
-            };
-            if (q.y > kUncappedOpacity) pixels(std::true_type{});
-            else pixels(std::false_type{});
-        }
-    }
-    if constexpr (kStats) {
-        if (G.px >= V.W) return;
-#pragma unroll
-        for (int p = 0; p < PX; p++) {
-            const int py = G.py0 + p;
-            if (py >= V.H) break;
-            const size_t pix = (size_t)py * V.W + G.px;
-            P.pix_neval[V.pix_base + pix] = neval[p];
-            P.pix_neval[P.total_pix + V.pix_base + pix] = nblend[p];
-        }
-    } else {
-        composite_epilogue<PX>(P, V, G, T, C0, C1, C2, D, O, last);
-        if (P.tile_walk) tile_walk_record<PX>(P, last);
-    }
-}
-
-// The compositor for an even number of pixels per thread, on packed pairs
-// of vertically adjacent pixels: the falloff, alpha, transmittance and
-// accumulation of both pixels of a pair take one .f32x2 instruction each.
-// The records are staged with their per-pixel operands duplicated into
-// pairs.  A pixel of a pair that does not blend (alpha < 1/255, stopped,
-// outside the image) adds a zero weight and keeps its T, which leaves its
-// sums bit-identical to skipping it, so the images equal the scalar
-// kernel's bit for bit.
-template <int TW, int TH, int PX>
-__global__ void __launch_bounds__(TW *TH / PX) k_composite_x2(Params P) {
+__global__ void __launch_bounds__(32, PX == 4 ? kFwdWarps4 : kFwdWarps2) k_composite(Params P) {
     pdl_enter();
     static_assert(PX % 2 == 0, "pairs of pixels");
-    constexpr int BLOCK = TW * TH / PX;
-    constexpr int NP = PX / 2;
+    constexpr int NP = PX / 2, U = kFwdUnroll;
     constexpr uint32_t ALL = (1u << PX) - 1u;
-    __shared__ float4 sA[BLOCK];  // (u, a', v, v)
-    __shared__ float4 sB[BLOCK];  // (b', b', c', c')
-    __shared__ float4 sC[BLOCK];  // (o~, o~, r, r)
-    __shared__ float4 sD[BLOCK];  // (g, g, b, b)
-    __shared__ float2 sE[BLOCK];  // (z, z)
-    const TileGeom G = tile_geom<TW, TH, PX>(P);
+    __shared__ RawRecords raw;
+    __shared__ Staged S;
+    const int lane = threadIdx.x;
+    const BlockGeom G = block_geom<PX>(P);
     const ViewDesc &V = *G.V;
     const uint2 r = G.r;
-    const int tid = threadIdx.x;
     const float fx = (float)G.px + 0.5f;
-    const float2 one2 = make_float2(1.0f, 1.0f);
+    const float2 nzero2 = make_float2(-0.0f, -0.0f);
     float2 fy[NP], T[NP], C0[NP], C1[NP], C2[NP], D[NP], O[NP];
-    uint32_t last[PX];
+    uint32_t last[PX];  // list position where the pixel stopped (else the list's length)
     uint32_t done = 0;
 #pragma unroll
     for (int q = 0; q < NP; q++) {
         fy[q] = make_float2((float)(G.py0 + 2 * q) + 0.5f, (float)(G.py0 + 2 * q + 1) + 0.5f);
-        T[q] = one2;
-        C0[q] = C1[q] = C2[q] = D[q] = O[q] = make_float2(0.f, 0.f);
+        T[q] = make_float2(1.0f, 1.0f);
+        C0[q] = C1[q] = C2[q] = D[q] = O[q] = nzero2;
     }
+    const uint32_t len = r.y - r.x;
 #pragma unroll
     for (int p = 0; p < PX; p++) {
-        last[p] = 0;
-        if (!(G.px < V.W && G.py0 + p < V.H)) done |= 1u << p;
+        last[p] = len;
+        if (!(G.px < V.W && G.py0 + p < V.H)) {
+            last[p] = 0;
+            done |= 1u << p;
+        }
     }
     // A pixel that is done (stopped, or outside the image) gets a row
     // coordinate far away: its falloff exponent is then -inf or NaN, its
-    // alpha 0 or NaN, and the alpha test (false for NaN) never passes
-    // again, so the loop needs no per-pixel done test.
+    // alpha 0 or NaN, and the alpha test (false for NaN) never passes again.
+    auto far_rows = [&]() {
 #pragma unroll
-    for (int q = 0; q < NP; q++) {
-        if (done & (1u << (2 * q))) fy[q].x = kFarRow;
-        if (done & (2u << (2 * q))) fy[q].y = kFarRow;
-    }
-    for (uint32_t base = r.x; base < r.y; base += BLOCK) {
-        if (__syncthreads_count(done != ALL) == 0) break;
-        const uint32_t j = base + tid;
-        if (j < r.y) {
-            float4 a, c;
-            float2 b;
-            record_terms(P.rec, P.pair_vals[j], a, b, c);
-            sA[tid] = make_float4(a.x, a.z, a.y, a.y);
-            sB[tid] = make_float4(a.w, a.w, b.x, b.x);
-            sC[tid] = make_float4(b.y, b.y, c.x, c.x);
-            sD[tid] = make_float4(c.y, c.y, c.z, c.z);
-            sE[tid] = make_float2(c.w, c.w);
+        for (int q = 0; q < NP; q++) {
+            if (done & (1u << (2 * q))) fy[q].x = kFarRow;
+            if (done & (2u << (2 * q))) fy[q].y = kFarRow;
         }
-        __syncthreads();
-        const int cnt = (int)min((uint32_t)BLOCK, r.y - base);
-        for (int k = 0; k < cnt && done != ALL; k++) {
-            const float4 A = sA[k], B = sB[k], Cq = sC[k], Dq = sD[k];
-            const float2 E = sE[k];
-            const uint32_t pos = base + k + 1 - r.x;  // list position after this entry
-            const float dx = __fsub_rn(fx, A.x);
-            const FalloffColumn fc = falloff_column(A.y, B.x, dx);
-            const float2 A2 = make_float2(fc.A, fc.A), B2 = make_float2(fc.B, fc.B);
-            const float2 v2 = make_float2(A.z, A.w), cp2 = make_float2(B.z, B.w);
-            const float2 o2 = make_float2(Cq.x, Cq.y), r2 = make_float2(Cq.z, Cq.w);
-            const float2 g2 = make_float2(Dq.x, Dq.y), b2 = make_float2(Dq.z, Dq.w);
-            // entries whose o~ cannot reach the cap skip min(cap, .)
-            auto pairs = [&](auto capped) {
-                constexpr bool kCap = decltype(capped)::value;
+    };
+    far_rows();
+    uint32_t m0 = lane < len ? P.pair_vals[r.x + lane] : kNoRecord;
+    fetch_record(P, raw, m0, lane);
+    uint32_t m1 = lane + 32u < len ? P.pair_vals[r.x + 32u + lane] : kNoRecord;
+    bool finished = __all_sync(0xffffffffu, done == ALL);
+    for (uint32_t base = 0; base < len && !finished; base += 32) {
+        wait_records();
+        const int hits = stage_hits<U>(raw, S, m0 != kNoRecord, m0, base + lane, G, lane);
+        m0 = m1;
+        fetch_record(P, raw, m0, lane);
+        m1 = base + 64u + lane < len ? P.pair_vals[r.x + base + 64u + lane] : kNoRecord;
+        for (int k = 0; k < hits; k += U) {
+            // alphas of U entries (negated, -0 where a pixel does not blend)
+            float2 na[U][NP];
+            uint32_t pos[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const float4 A = S.a[k + u], B = S.b[k + u];
+                const float2 no2 = reinterpret_cast<const float2 *>(&S.c[k + u])[0];
+                pos[u] = __float_as_uint(A.w);
+                const float dx = __fsub_rn(fx, A.x);
+                const FalloffColumn fc = falloff_column(A.y, A.z, dx);
+                const float2 A2 = make_float2(fc.A, fc.A), B2 = make_float2(fc.B, fc.B);
+                const float2 v2 = make_float2(B.x, B.y), cp2 = make_float2(B.z, B.w);
 #pragma unroll
                 for (int q = 0; q < NP; q++) {
-                    const float2 dy = sub2(fy[q], v2);
-                    const float2 e = falloff_exp2_x2(A2, B2, cp2, dy);
-                    const float2 a = mul2(o2, make_float2(ex2_approx(e.x), ex2_approx(e.y)));
-                    // min(cap, a) >= 1/255 iff a >= 1/255 (cap > 1/255): the cap
-                    // is applied to blending pixels only
-                    // a done pixel (far row, c' <= -kMinRowCoef) has alpha 0
-                    bool bx = a.x >= kAlphaMin, by = a.y >= kAlphaMin;
-                    if (!(bx || by)) continue;
-                    const float ax = kCap ? fminf(kAlphaCap, a.x) : a.x, ay = kCap ? fminf(kAlphaCap, a.y) : a.y;
-                    const float2 al = make_float2(ax, ay);
-                    const float2 wu = mul2(al, T[q]);
-                    const float2 Tn = sub2(T[q], wu);
-                    const bool sx = bx && Tn.x < kTStop, sy = by && Tn.y < kTStop;
-                    if (sx || sy) {
-                        done |= ((sx ? 1u : 0u) | (sy ? 2u : 0u)) << (2 * q);
-                        if (sx) fy[q].x = kFarRow;
-                        if (sy) fy[q].y = kFarRow;
-                    }
-                    bx = bx && !sx;
-                    by = by && !sy;
-                    // a pixel that does not blend takes w = +0 and T - 0 = T, bit
-                    // for bit; a blending one gets the scalar kernel's w and T'
-                    const float2 w = make_float2(bx ? wu.x : 0.f, by ? wu.y : 0.f);
-                    C0[q] = fma2(r2, w, C0[q]);
-                    C1[q] = fma2(g2, w, C1[q]);
-                    C2[q] = fma2(b2, w, C2[q]);
-                    D[q] = fma2(E, w, D[q]);
-                    O[q] = add2(O[q], w);
-                    T[q] = sub2(T[q], w);
-                    last[2 * q] = bx ? pos : last[2 * q];
-                    last[2 * q + 1] = by ? pos : last[2 * q + 1];
+                    const float2 e = falloff_exp2_x2(A2, B2, cp2, sub2(fy[q], v2));
+                    const float2 nr = mul2(no2, make_float2(ex2_approx(e.x), ex2_approx(e.y)));
+                    na[u][q] = make_float2(nr.x <= -kAlphaMin ? nr.x : -0.0f, nr.y <= -kAlphaMin ? nr.y : -0.0f);
                 }
-            };
-            if (Cq.x > kUncappedOpacity) pairs(std::true_type{});
-            else pairs(std::false_type{});
+            }
+            uint32_t flags = pos[0];
+#pragma unroll
+            for (int u = 1; u < U; u++) flags |= pos[u];
+            if (flags > kPosMask) {
+                // o~ may exceed the cap (one that cannot is left as it is)
+#pragma unroll
+                for (int u = 0; u < U; u++)
+#pragma unroll
+                    for (int q = 0; q < NP; q++)
+                        na[u][q] = make_float2(fmaxf(na[u][q].x, -kAlphaCap), fmaxf(na[u][q].y, -kAlphaCap));
+                if (flags & kOddEntry) {  // non-finite terms: one pixel at a time
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        const float col[4] = {S.c[k + u].z, S.d[k + u].x, S.d[k + u].z, S.e[k + u].x};
+                        auto one = [&](float nal, float &t, float &c0, float &c1, float &c2, float &d, float &o, int p) {
+                            if (!(nal < 0.0f) || (done & (1u << p))) return;
+                            const float nw = __fmul_rn(nal, t), tn = __fadd_rn(t, nw);
+                            if (tn < kTStop) {
+                                done |= 1u << p;
+                                last[p] = pos[u] & kPosMask;
+                                return;
+                            }
+                            c0 = __fmaf_rn(col[0], nw, c0);
+                            c1 = __fmaf_rn(col[1], nw, c1);
+                            c2 = __fmaf_rn(col[2], nw, c2);
+                            d = __fmaf_rn(col[3], nw, d);
+                            o = __fadd_rn(o, nw);
+                            t = tn;
+                        };
+#pragma unroll
+                        for (int q = 0; q < NP; q++) {
+                            one(na[u][q].x, T[q].x, C0[q].x, C1[q].x, C2[q].x, D[q].x, O[q].x, 2 * q);
+                            one(na[u][q].y, T[q].y, C0[q].y, C1[q].y, C2[q].y, D[q].y, O[q].y, 2 * q + 1);
+                        }
+                    }
+                    far_rows();
+                    if (__all_sync(0xffffffffu, done == ALL)) {
+                        finished = true;
+                        break;
+                    }
+                    continue;
+                }
+            }
+            // weights; T only falls, so a pixel stops in these entries exactly
+            // if its T after the last of them is below the stop
+            float2 nw[U][NP], Tn[NP];
+            bool stop = false;
+#pragma unroll
+            for (int q = 0; q < NP; q++) {
+                Tn[q] = T[q];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    nw[u][q] = mul2(na[u][q], Tn[q]);
+                    Tn[q] = add2(Tn[q], nw[u][q]);
+                }
+                stop |= Tn[q].x < kTStop || Tn[q].y < kTStop;
+            }
+            const bool any_stop = __any_sync(0xffffffffu, stop);
+            if (any_stop) {
+                // a pixel takes no part from the entry that would stop it on
+                auto stopping = [&](float t, float &tn, auto weight, int p) {
+                    if (!(tn < kTStop)) return;
+                    bool off = false;
+#pragma unroll
+                    for (int u = 0; u < U; u++) {
+                        float &w = weight(u);
+                        if (!off && __fadd_rn(t, w) < kTStop) {
+                            off = true;
+                            done |= 1u << p;
+                            last[p] = pos[u] & kPosMask;
+                        }
+                        if (off) w = -0.0f;
+                        t = __fadd_rn(t, w);
+                    }
+                    tn = t;
+                };
+#pragma unroll
+                for (int q = 0; q < NP; q++) {
+                    stopping(T[q].x, Tn[q].x, [&](int u) -> float & { return nw[u][q].x; }, 2 * q);
+                    stopping(T[q].y, Tn[q].y, [&](int u) -> float & { return nw[u][q].y; }, 2 * q + 1);
+                }
+                far_rows();
+            }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const float2 r2 = reinterpret_cast<const float2 *>(&S.c[k + u])[1], z2 = S.e[k + u];
+                const float4 Dq = S.d[k + u];
+                const float2 g2 = make_float2(Dq.x, Dq.y), b2 = make_float2(Dq.z, Dq.w);
+#pragma unroll
+                for (int q = 0; q < NP; q++) {
+                    C0[q] = fma2(r2, nw[u][q], C0[q]);
+                    C1[q] = fma2(g2, nw[u][q], C1[q]);
+                    C2[q] = fma2(b2, nw[u][q], C2[q]);
+                    D[q] = fma2(z2, nw[u][q], D[q]);
+                    O[q] = add2(O[q], nw[u][q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < NP; q++) T[q] = Tn[q];
+            if (any_stop && __all_sync(0xffffffffu, done == ALL)) {
+                finished = true;
+                break;
+            }
         }
+        __syncwarp();  // the next group restages
     }
+    wait_records();  // a copy may still be under way when the walk ended early
     float Ts[PX], C0s[PX], C1s[PX], C2s[PX], Ds[PX], Os[PX];
 #pragma unroll
     for (int q = 0; q < NP; q++) {
         Ts[2 * q] = T[q].x; Ts[2 * q + 1] = T[q].y;
-        C0s[2 * q] = C0[q].x; C0s[2 * q + 1] = C0[q].y;
-        C1s[2 * q] = C1[q].x; C1s[2 * q + 1] = C1[q].y;
-        C2s[2 * q] = C2[q].x; C2s[2 * q + 1] = C2[q].y;
-        Ds[2 * q] = D[q].x; Ds[2 * q + 1] = D[q].y;
-        Os[2 * q] = O[q].x; Os[2 * q + 1] = O[q].y;
+        C0s[2 * q] = -C0[q].x; C0s[2 * q + 1] = -C0[q].y;
+        C1s[2 * q] = -C1[q].x; C1s[2 * q + 1] = -C1[q].y;
+        C2s[2 * q] = -C2[q].x; C2s[2 * q + 1] = -C2[q].y;
+        Ds[2 * q] = -D[q].x; Ds[2 * q + 1] = -D[q].y;
+        Os[2 * q] = -O[q].x; Os[2 * q + 1] = -O[q].y;
     }
     composite_epilogue<PX>(P, V, G, Ts, C0s, C1s, C2s, Ds, Os, last);
-    if (P.tile_walk) tile_walk_record<PX>(P, last);
+    if (P.tile_walk) {  // how far the tile's adjoint walks, for its launch order
+        uint32_t w = last[0];
+#pragma unroll
+        for (int p = 1; p < PX; p++) w = max(w, last[p]);
+        w = __reduce_max_sync(0xffffffffu, w);
+        if (lane == 0 && w) atomicMax(&P.tile_walk[G.tile], w);
+    }
 }
 
-template <int TW, int TH, int PX>
-void launch_fwd_t(const Params &p, cudaStream_t s) {
-    note_launch();
-    if constexpr (PX % 2 == 0)
-        pdl_launch(k_composite_x2<TW, TH, PX>, p.total_tiles, TW * TH / PX, 0, s, p);
-    else
-        pdl_launch(k_composite<TW, TH, PX, false>, p.total_tiles, TW * TH / PX, 0, s, p);
-}
-
-template <int TW, int TH, int PX>
-void launch_stats_t(const Params &p, cudaStream_t s) {
-    note_launch();
-    pdl_launch(k_composite<TW, TH, PX, true>, p.total_tiles, TW * TH / PX, 0, s, p);
+// Work counts of the last forward, one pixel per thread: the number of list
+// entries whose footprint box contains the pixel, up to and including the
+// one that stopped it (the compositing work E), and the number of those with
+// alpha >= 1/255 (blended, or stopping the pixel).
+__global__ void __launch_bounds__(32) k_composite_stats(Params P) {
+    pdl_enter();
+    const BlockGeom G = block_geom<1>(P);
+    const ViewDesc &V = *G.V;
+    if (!(G.px < V.W && G.py0 < V.H)) return;
+    const float fx = (float)G.px + 0.5f, fy = (float)G.py0 + 0.5f;
+    float T = 1.0f;
+    uint32_t neval = 0, nblend = 0;
+    for (uint32_t j = G.r.x; j < G.r.y; j++) {
+        const uint32_t m = P.pair_vals[j];
+        float4 g, col;
+        float2 q;
+        record_terms(P.rec, m, g, q, col);
+        const float dx = __fsub_rn(fx, g.x), dy = __fsub_rn(fy, g.y);
+        if (fabsf(dx) <= P.rec[3 * (size_t)m + 1].w && fabsf(dy) <= P.rec[3 * (size_t)m + 2].w) neval++;
+        const float raw = __fmul_rn(q.y, ex2_approx(falloff_exp2(falloff_column(g.z, g.w, dx), q.x, dy)));
+        if (!(raw >= kAlphaMin)) continue;
+        nblend++;
+        const float Tn = __fsub_rn(T, __fmul_rn(fminf(kAlphaCap, raw), T));
+        if (Tn < kTStop) break;
+        T = Tn;
+    }
+    const size_t pix = (size_t)G.py0 * V.W + G.px;
+    P.pix_neval[V.pix_base + pix] = neval;
+    P.pix_neval[P.total_pix + V.pix_base + pix] = nblend;
 }
 
 }  // namespace
@@ -334,19 +322,43 @@ bool composite_supported(int tw, int th, int px) {
     return false;
 }
 
-#define PVG_DISPATCH_ONE_fwd(W, H, X) \
-    if (p.tile_w == W && p.tile_h == H && p.px == X) return launch_fwd_t<W, H, X>(p, s);
-#define PVG_DISPATCH_ONE_stats(W, H, X) \
-    if (p.tile_w == W && p.tile_h == H && p.px == X) return launch_stats_t<W, H, X>(p, s);
+// Pixels per lane and block shape of the compositing kernels.  More pixels
+// per lane share an entry's work among more pixels; fewer make more and
+// shorter walks, which a frame that cannot fill the SMs with wide blocks (or
+// a tile of 64 pixels) needs.
+WarpShape warp_shape(const Params &p, int wide4, int wide8) {
+    const int pixels = p.tile_w * p.tile_h;
+    const int64_t all = (int64_t)p.total_tiles * pixels, sms = device_sm_count();
+    WarpShape w;
+    w.px = p.tile_w >= 16 && p.tile_h >= 16 && all / 256 >= wide8 * sms ? 8
+           : pixels >= 128 && all / 128 >= wide4 * sms                  ? 4
+                                                                        : 2;
+    w.shift = w.px == 8 || (w.px == 4 && p.tile_h < 16) ? 4 : 3;
+    w.blocks = (uint32_t)(pixels / (32 * w.px));
+    return w;
+}
+
+static Params with_shape(const Params &p, const WarpShape &w) {
+    Params q = p;
+    q.block_shift = w.shift;
+    q.blocks_per_tile = w.blocks;
+    return q;
+}
 
 void launch_composite(const Params &p, cudaStream_t s) {
     if (p.total_tiles == 0) return;
-    PVG_TILE_CONFIGS(PVG_DISPATCH_ONE_fwd)
+    const WarpShape w = warp_shape(p, kFwdWide, INT_MAX);
+    const Params q = with_shape(p, w);
+    note_launch();
+    if (w.px == 4) pdl_launch(k_composite<4>, p.total_tiles * w.blocks, 32, 0, s, q);
+    else pdl_launch(k_composite<2>, p.total_tiles * w.blocks, 32, 0, s, q);
 }
 
 void launch_composite_stats(const Params &p, cudaStream_t s) {
     if (p.total_tiles == 0) return;
-    PVG_TILE_CONFIGS(PVG_DISPATCH_ONE_stats)
+    const Params q = with_shape(p, WarpShape{1, 3, (uint32_t)(p.tile_w * p.tile_h / 32)});
+    note_launch();
+    pdl_launch(k_composite_stats, p.total_tiles * q.blocks_per_tile, 32, 0, s, q);
 }
 
 }  // namespace pvg

@@ -1,21 +1,18 @@
 // raster_bwd.cu -- adjoint of the per-tile compositing (stage d1).
 //
-// The compositor's CTA shape walks the tile's list back to front from the
-// last blended position of any pixel, rebuilding T_i = T_{i+1} / (1 -
-// alpha_i).  With X_i = gC.c_i + gD z_i + gO (the pixel's output gradients
-// against entry i's channels) and the scalar suffix sum
+// A warp walks its block's hits (raster_common.cuh) back to front from the
+// last position any of its pixels takes part in, rebuilding T_i = T_{i+1} /
+// (1 - alpha_i).  With X_i = gC.c_i + gD z_i + gO (the pixel's output
+// gradients against entry i's channels) and the scalar suffix sum
 //   S_i = sum_{j > i} X_j alpha_j T_j  (+ T_final gC.bg),
 // the derivative of the pixel's loss with respect to alpha_i is
 //   dL/dalpha_i = T_i X_i - S_i / (1 - alpha_i),
 // so one scalar per pixel carries what the colour, depth and opacity
-// suffix sums would.  The 10 image-space gradient terms of an entry
-// (moments of dL/dpower for u, v, conic a b c; o~; r g b; z) are summed
-// over a thread's PX pixels, then over the warp by transposing butterflies
-// (afterwards lane s holds term s), added to
-// per-CTA shared accumulators by 10 lanes at once, and reach global memory with one
-// atomic per (Gaussian, tile, term).  Alpha is the forward's expression
-// (explicit roundings), so the blend decisions are the forward's; the rest
-// of this file may contract a*b+c into fused multiply-adds.
+// suffix sums would.  The image-space gradient terms of an entry (moments of
+// dL/dpower; r g b; z) are summed over a lane's pixels, then over the warp
+// (flush_terms) and added to the Gaussian's row in global memory.  Alpha is the forward's expression (explicit roundings), so the
+// blend decisions are the forward's; the rest of this file may contract
+// a*b+c into fused multiply-adds.
 #include <type_traits>
 
 #include "raster_common.cuh"
@@ -23,47 +20,100 @@
 namespace pvg {
 namespace {
 
-// Sum of v[0..NT-1] (NT = 9 or 10) over the warp, as transposing
-// butterflies: terms 0..7 within groups of 8 lanes (4 + 2 + 1 exchanges,
-// then two folds across the groups); for NT = 10 terms 8, 9 between lane
-// pairs (1 exchange, four folds), for NT = 9 term 8 by a plain butterfly.
-// On return lane L holds in .x the total of term L & 7 and in .y that of
-// term 8 + (L & 1) (NT = 10) or term 8 (NT = 9); lanes 0..NT-1 therefore
-// hold term L in .x (L < 8) or .y.  12 shuffles and 44 instructions for
-// NT = 10 instead of one 16-slot butterfly's 62.
+// Resident warps per SM that the registers are held to (no spills: 16 warps
+// of 126 registers with eight pixels per lane), and entries whose alphas are
+// evaluated together, by pixels per lane: with two pixels a lane the walk is
+// latency-bound and overlaps four, with eight the pixels are parallel enough.
+template <int PX>
+struct BwdTune {
+    static constexpr int kWarps = PX == 2 ? 20 : 16;
+    static constexpr int kUnroll = PX == 8 ? 1 : PX == 4 ? 2 : 4;
+};
+// Blocks of 256 (128) pixels per SM from which a lane takes eight (four)
+// pixels.  Eight make an entry's fixed work (its staged loads, the warp sum,
+// the atomics) a quarter of that of two: 362 us against 405 us with four on
+// the 1.5M-Gaussian 1920x1280 frame (9,600 blocks), 2.15 against 2.38 ms on
+// 12 mixed views (14,900 blocks); a 961x641 frame of 300k Gaussians (2,501
+// blocks), which its longest walks bound, takes 535 us with eight, 291 us
+// with four.  Two only for frames too small for four (1242x375: 178 us with
+// two, 133 us with four).
+constexpr int kBwdWide8 = 48, kBwdWide4 = 16;
+
+// Warp sums of an entry's NT terms (9, or 10 with the depth term) over the
+// lanes, four entries at a time, by a transposition through shared memory:
+// every lane stores its terms of an entry (two float4 and one or two
+// floats), and once four entries are stored lane r sums eight lanes' float4
+// of entry r >> 3, half (r >> 2) & 1, and folds the four partial sums that
+// the lanes r & 3 of a half hold with three shuffles.  About 14 instructions
+// per entry; a shuffle butterfly over 9 terms takes 44.  The halves are 36
+// float4 apart so that the eight lanes of a load phase (two halves, four
+// lanes each) read distinct banks.
+constexpr int kSlots = 4;
+constexpr int kHalfStride = 36;
+
 template <int NT>
-__device__ __forceinline__ float2 warp_sum_terms(const float (&v)[10]) {
-    static_assert(NT == 9 || NT == 10, "9 or 10 terms");
-    const int lane = threadIdx.x & 31;
-    bool hi = lane & 4;
-    float b[4];
+struct TermBuffer {
+    float4 h[kSlots][2][kHalfStride];
+    float e[NT - 8][kSlots][32];
+};
+
+// Adds the totals of the stored entries (bit i of `valid`: slot i, staged
+// entry base + i) to their Gaussians' rows.
+template <int NT>
+__device__ __forceinline__ void flush_terms(const TermBuffer<NT> &buf, const Staged &S, int base, uint32_t valid,
+                                            int lane, const Params &P) {
+    __syncwarp();
+    const int slot = lane >> 3, half = (lane >> 2) & 1, sub = lane & 3;
+    const float4 *h = &buf.h[slot][half][sub];
+    float2 a, b;
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
-        const float send = hi ? v[i] : v[i + 4];
-        b[i] = (hi ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, send, 4);
+    for (int j = 0; j < 8; j++) {
+        const float4 v = h[4 * j];
+        a = j ? add2(a, make_float2(v.x, v.y)) : make_float2(v.x, v.y);
+        b = j ? add2(b, make_float2(v.z, v.w)) : make_float2(v.z, v.w);
     }
-    hi = lane & 2;
-    float c[2];
+    const bool hi2 = sub & 2, hi1 = sub & 1;
+    const float c0 = (hi2 ? b.x : a.x) + __shfl_xor_sync(0xffffffffu, hi2 ? a.x : b.x, 2);
+    const float c1 = (hi2 ? b.y : a.y) + __shfl_xor_sync(0xffffffffu, hi2 ? a.y : b.y, 2);
+    float d = (hi1 ? c1 : c0) + __shfl_xor_sync(0xffffffffu, hi1 ? c0 : c1, 1);
+    float s[NT - 8];
 #pragma unroll
-    for (int i = 0; i < 2; i++) {
-        const float send = hi ? b[i] : b[i + 2];
-        c[i] = (hi ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, send, 2);
+    for (int t = 0; t < NT - 8; t++) {
+        const float4 v = reinterpret_cast<const float4 *>(&buf.e[t][0][0])[lane];
+        s[t] = (v.x + v.y) + (v.z + v.w);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) s[t] += __shfl_xor_sync(0xffffffffu, s[t], o);
     }
-    hi = lane & 1;
-    float d = (hi ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, hi ? c[0] : c[1], 1);
-    d += __shfl_xor_sync(0xffffffffu, d, 8);
-    d += __shfl_xor_sync(0xffffffffu, d, 16);
-    float e;
-    if constexpr (NT == 10) {
-        e = (hi ? v[9] : v[8]) + __shfl_xor_sync(0xffffffffu, hi ? v[8] : v[9], 1);
-#pragma unroll
-        for (int o = 2; o < 32; o <<= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-    } else {
-        e = v[8];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    // half 0 holds m_xx, m_xy, m_yy, m_0, half 1 m_x, m_y, r, g
+    const float q = __shfl_xor_sync(0xffffffffu, d, 1);
+    if ((valid >> slot) & 1u) {
+        const size_t m = S.m[base + slot];
+        const float4 gb = S.d[base + slot], ab = S.a[base + slot];
+        if (half == 0 && sub < 3) {
+            // the second moments in 64 bits: the per-item adjoint's products
+            // with the conic cancel and amplify the rounding of their sums
+            if (d != 0.f) atomicAdd(P.g2m + 3 * m + sub, (double)d);
+        } else {
+            bool keep = d != 0.f;
+            int t = kG2dColour + sub - 2;
+            if (half == 0) {
+                t = kG2dPower;
+            } else if (sub < 2) {
+                // gradients of u and v (conic a = -2 ln 2 a', b = -ln 2 b'),
+                // here and not from the moments' totals: a m_x + b m_y cancels
+                const float own = sub == 0 ? ab.y : S.b[base + slot].z;
+                d = -0.6931471805599453f * (2.0f * own * d + ab.z * q);
+                keep = d != 0.f;
+                t = sub;
+            } else {  // the colours: none where the forward clamped
+                keep = keep && (sub == 2 ? S.c[base + slot].z : gb.x) > 0.f;
+            }
+            if (keep) atomicAdd(P.g2d + kG2dRow * m + t, d);
+        }
+        if ((lane & 7) == 0 && s[0] != 0.f && gb.z > 0.f) atomicAdd(P.g2d + kG2dRow * m + kG2dColour + 2, s[0]);
+        if (NT == 10 && (lane & 7) == 1 && s[NT - 9] != 0.f) atomicAdd(P.g2d + kG2dRow * m + kG2dDepth, s[NT - 9]);
     }
-    return make_float2(d, e);
+    __syncwarp();
 }
 
 // Per-pixel state of the adjoint walk: final transmittance, last blended
@@ -117,174 +167,212 @@ __device__ __forceinline__ PixelAdjoint pixel_adjoint(const Params &P, const Vie
     return a;
 }
 
-// Image-space gradients of a staged entry from its CTA-summed terms:
-//   d/da = -m_xx / 2, d/db = -m_xy, d/dc = -m_yy / 2,
-//   d/du = (a m_x + b m_y) = -(2 a' m_x + b' m_y) / log2(e),
-//   d/dv = (b m_x + c m_y) = -(b' m_x + 2 c' m_y) / log2(e);
-// colour terms are zeroed where the forward clamped (col <= 0).
-__device__ __forceinline__ void flush_entry(float *dst, const float *a, float ap, float bp, float cp, float r,
-                                            float g, float b) {
-    float gt[10];
-    gt[0] = -0.6931471805599453f * (2.f * ap * a[0] + bp * a[1]);
-    gt[1] = -0.6931471805599453f * (bp * a[0] + 2.f * cp * a[1]);
-    gt[2] = -0.5f * a[2];
-    gt[3] = -a[3];
-    gt[4] = -0.5f * a[4];
-    gt[5] = a[5];
-    gt[6] = r > 0.f ? a[6] : 0.f;
-    gt[7] = g > 0.f ? a[7] : 0.f;
-    gt[8] = b > 0.f ? a[8] : 0.f;
-    gt[9] = a[9];
-#pragma unroll
-    for (int c = 0; c < 10; c++)
-        if (gt[c] != 0.f) atomicAdd(dst + c, gt[c]);
-}
-
 // kAux: the call has depth or opacity-map gradients or a sky map (dL/dO
 // and the depth term of X can be non-zero); without them X = gC.c and the
-// depth term is not reduced (9 terms).
-template <int TW, int TH, int PX, bool kAux>
-__global__ void __launch_bounds__(TW *TH / PX) k_composite_bwd(Params P) {
+// depth term is not reduced (9 terms).  The output gradients and the blend
+// weights are kept negated, which leaves the packed arithmetic no negation.
+template <int PX, bool kAux>
+__global__ void __launch_bounds__(32, BwdTune<PX>::kWarps) k_composite_bwd(Params P) {
     pdl_enter();
-    constexpr int BLOCK = TW * TH / PX;
-    constexpr int NG = 10;               // shared accumulator stride
-    constexpr int NT = kAux ? 10 : 9;    // terms reduced
-    __shared__ float4 s0[BLOCK];
-    __shared__ float2 s1[BLOCK];
-    __shared__ float4 s2[BLOCK];
-    __shared__ uint32_t s_m[BLOCK];
-    __shared__ float s_acc[BLOCK * NG];
-    __shared__ uint32_t s_maxlast;
-    const TileGeom Gm = tile_geom<TW, TH, PX>(P);
-    const ViewDesc &V = *Gm.V;
-    const uint2 r = Gm.r;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const float fx = (float)Gm.px + 0.5f;
-
-    float fy[PX], T[PX], gC0[PX], gC1[PX], gC2[PX], gD[PX], gO[PX];
-    float S[PX];  // suffix sum of X_j alpha_j T_j
+    constexpr int NT = kAux ? 10 : 9, NP = PX / 2, U = BwdTune<PX>::kUnroll;
+    __shared__ RawRecords raw;
+    __shared__ Staged Sg;
+    __shared__ TermBuffer<NT> buf;
+    const int lane = threadIdx.x;
+    const BlockGeom G = block_geom<PX>(P);
+    const ViewDesc &V = *G.V;
+    const uint2 r = G.r;
+    const float fx = (float)G.px + 0.5f;
+    const float2 one2 = make_float2(1.0f, 1.0f);
+    float2 fy[NP], T[NP], nC0[NP], nC1[NP], nC2[NP], nD[NP], nO[NP];
+    float2 S[NP];  // suffix sum of X_j alpha_j T_j
     uint32_t last[PX];
-    uint32_t maxlast = 0;
+    uint32_t walk = 0;
+    bool odd = false;  // non-finite or huge output gradients: pixels one at a time
 #pragma unroll
-    for (int p = 0; p < PX; p++) {
-        fy[p] = (float)(Gm.py0 + p) + 0.5f;
-        PixelAdjoint a = pixel_adjoint(P, V, Gm.px, Gm.py0 + p);
-        T[p] = a.T; last[p] = a.last; S[p] = a.S;
-        gC0[p] = a.gC0; gC1[p] = a.gC1; gC2[p] = a.gC2; gD[p] = a.gD; gO[p] = a.gO;
-        maxlast = max(maxlast, last[p]);
+    for (int q = 0; q < NP; q++) {
+        fy[q] = make_float2((float)(G.py0 + 2 * q) + 0.5f, (float)(G.py0 + 2 * q + 1) + 0.5f);
+        const PixelAdjoint a = pixel_adjoint(P, V, G.px, G.py0 + 2 * q), b = pixel_adjoint(P, V, G.px, G.py0 + 2 * q + 1);
+        T[q] = make_float2(a.T, b.T);
+        S[q] = make_float2(a.S, b.S);
+        nC0[q] = make_float2(-a.gC0, -b.gC0);
+        nC1[q] = make_float2(-a.gC1, -b.gC1);
+        nC2[q] = make_float2(-a.gC2, -b.gC2);
+        nD[q] = make_float2(-a.gD, -b.gD);
+        nO[q] = make_float2(-a.gO, -b.gO);
+        last[2 * q] = a.last;
+        last[2 * q + 1] = b.last;
+        walk = max(walk, max(a.last, b.last));
+        for (const PixelAdjoint &e : {a, b})
+            odd |= !(fabsf(e.gC0) + fabsf(e.gC1) + fabsf(e.gC2) + fabsf(e.gD) + fabsf(e.gO) + fabsf(e.S) < 1e15f);
     }
-    if (tid == 0) s_maxlast = 0;
-    __syncthreads();
-    if (maxlast) atomicMax(&s_maxlast, maxlast);
-    __syncthreads();
-    const uint32_t n = s_maxlast;
-    // gv: an entry's 10 terms over this thread's pixels, zero between
-    // entries (reset after each warp reduction).  The pixels share dx, so
-    // the conic moments are kept as sum gpow (A0), sum gpow dy (gv[1]) and
-    // sum gpow dy^2 (gv[4]) and expanded once: m_x = dx A0, m_xx = dx^2 A0,
-    // m_xy = dx m_y.
-    float gv[NG];
+    odd = __any_sync(0xffffffffu, odd);
+    walk = __reduce_max_sync(0xffffffffu, walk);
+    // groups of 32 entries from the walk's end; lane i of a group holds entry start + i
+    auto load_index = [&](int start) { return start + lane >= 0 && start + lane < (int)walk ? P.pair_vals[r.x + start + lane] : kNoRecord; };
+    int start = (int)walk - 32;
+    uint32_t m0 = load_index(start);
+    fetch_record(P, raw, m0, lane);
+    uint32_t m1 = load_index(start - 32);
+    for (; start > -32; start -= 32) {
+        wait_records();
+        const int hits = stage_hits<kSlots>(raw, Sg, m0 != kNoRecord, m0, (uint32_t)(start + lane), G, lane);
+        m0 = m1;
+        fetch_record(P, raw, m0, lane);
+        m1 = load_index(start - 64);
+        for (int base = (hits - 1) & ~(kSlots - 1); base >= 0; base -= kSlots) {
+            uint32_t valid = 0;  // slots that hold an entry's terms
+#pragma unroll 1
+            for (int k0 = kSlots - U; k0 >= 0; k0 -= U) {
+                // alphas of U entries, the later first (negated, 0 where a pixel does not blend)
+                float2 dy[U][NP], na[U][NP];
+                float dx[U];
+                uint32_t pf[U];
+                uint32_t any = 0;
 #pragma unroll
-    for (int c = 0; c < NG; c++) gv[c] = 0.f;
-    float A0 = 0.f;
-    for (uint32_t end = r.x + n; end > r.x;) {
-        const uint32_t start = end - r.x > (uint32_t)BLOCK ? end - BLOCK : r.x;
-        const int cnt = (int)(end - start);
-        __syncthreads();
-        if (tid < cnt) {
-            const uint32_t m = P.pair_vals[start + tid];
-            stage_record(P, m, s0, s1, s2, tid);
-            s_m[tid] = m;
-        }
-        for (int k = tid; k < BLOCK * NG; k += BLOCK) s_acc[k] = 0.f;
-        __syncthreads();
-        for (int k = cnt - 1; k >= 0; k--) {
-            const uint32_t pos = start + k - r.x;  // list position
-            bool contrib = false;
-            if (pos < maxlast) {  // before the last blend of one of this thread's pixels
-                const float4 g = s0[k];
-                const float2 q = s1[k];
-                const float4 col = s2[k];
-                const float dx = __fsub_rn(fx, g.x);
-                const FalloffColumn fc = falloff_column(g.z, g.w, dx);
-                // entries whose o~ cannot reach the cap skip min(cap, .)
-                auto pixels = [&](auto capped) {
-                    constexpr bool kCap = decltype(capped)::value;
+                for (int u = U - 1; u >= 0; u--) {
+                    const int k = base + k0 + u;
+                    const float4 A = Sg.a[k], B = Sg.b[k];
+                    const float2 no2 = reinterpret_cast<const float2 *>(&Sg.c[k])[0];
+                    pf[u] = __float_as_uint(A.w);
+                    const uint32_t pos = pf[u] & kPosMask;
+                    dx[u] = __fsub_rn(fx, A.x);
+                    const FalloffColumn fc = falloff_column(A.y, A.z, dx[u]);
+                    const float2 A2 = make_float2(fc.A, fc.A), B2 = make_float2(fc.B, fc.B);
+                    const float2 v2 = make_float2(B.x, B.y), cp2 = make_float2(B.z, B.w);
+                    bool hit = false;
 #pragma unroll
-                    for (int p = 0; p < PX; p++) {
-                        if (pos >= last[p]) continue;
-                        const float dy = __fsub_rn(fy[p], g.y);
-                        const float e = falloff_exp2(fc, q.x, dy);
-                        const float G = ex2_approx(e);
-                        const float raw = __fmul_rn(q.y, G);
-                        if (!(raw >= kAlphaMin)) continue;  // = min(cap, raw) < 1/255, cap > 1/255
-                        const float alpha = kCap ? fminf(kAlphaCap, raw) : raw;
-                        contrib = true;
-                        const float inv = rcp_approx(1.0f - alpha);
-                        const float Ti = T[p] * inv;
-                        const float w = alpha * Ti;
-                        float X = gC0[p] * col.x + gC1[p] * col.y + gC2[p] * col.z;
-                        if constexpr (kAux) X += gD[p] * col.w + gO[p];
-                        const float ga = Ti * X - inv * S[p];
-                        gv[6] += gC0[p] * w;
-                        gv[7] += gC1[p] * w;
-                        gv[8] += gC2[p] * w;
-                        if constexpr (kAux) gv[9] += gD[p] * w;
-                        if (!kCap || raw <= kAlphaCap) {
-                            // moments of gpow = dL/dpower (d alpha / d power = alpha);
-                            // the conic is applied once per Gaussian in the flush
-                            gv[5] += ga * G;
-                            const float gpow = ga * alpha;
-                            const float my = gpow * dy;
-                            A0 += gpow;
-                            gv[1] += my;
-                            gv[4] += my * dy;
-                        }
-                        S[p] += X * w;
-                        T[p] = Ti;
+                    for (int q = 0; q < NP; q++) {
+                        dy[u][q] = sub2(fy[q], v2);
+                        const float2 e = falloff_exp2_x2(A2, B2, cp2, dy[u][q]);
+                        const float2 nr = mul2(no2, make_float2(ex2_approx(e.x), ex2_approx(e.y)));
+                        const bool bx = pos < last[2 * q] && nr.x <= -kAlphaMin;
+                        const bool by = pos < last[2 * q + 1] && nr.y <= -kAlphaMin;
+                        hit |= bx || by;
+                        na[u][q] = make_float2(bx ? nr.x : 0.f, by ? nr.y : 0.f);
                     }
-                };
-                if (q.y > kUncappedOpacity) pixels(std::true_type{});
-                else pixels(std::false_type{});
-                if (contrib) {
-                    gv[0] = dx * A0;
-                    gv[2] = dx * gv[0];
-                    gv[3] = dx * gv[1];
+                    any |= __any_sync(0xffffffffu, hit) ? 1u << u : 0u;
                 }
-            }
-            if (__any_sync(0xffffffffu, contrib)) {
-                const float2 tot = warp_sum_terms<NT>(gv);
-                if (lane < NT) atomicAdd(&s_acc[k * NG + lane], lane < 8 ? tot.x : tot.y);
 #pragma unroll
-                for (int c = 0; c < NG; c++) gv[c] = 0.f;
-                A0 = 0.f;
+                for (int u = U - 1; u >= 0; u--) {
+                    if (!((any >> u) & 1u)) continue;
+                    const int k = base + k0 + u;
+                    const float2 r2 = reinterpret_cast<const float2 *>(&Sg.c[k])[1];
+                    const float4 Dq = Sg.d[k];
+                    const float2 g2 = make_float2(Dq.x, Dq.y), b2 = make_float2(Dq.z, Dq.w);
+                    float2 z2;
+                    if constexpr (kAux) z2 = Sg.e[k];
+                    float A0, M1, M2, c0, c1, c2, zs = 0.f;
+                    if (!odd && !(pf[u] & kOddEntry)) {
+                        float2 A0v, M1v, M2v, c0v, c1v, c2v, zv;
+                        auto pairs = [&](auto capped) {
+                            constexpr bool kCap = decltype(capped)::value;
+#pragma unroll
+                            for (int q = 0; q < NP; q++) {
+                                float2 nq = na[u][q];
+                                bool ox = false, oy = false;  // over the cap: alpha does not depend on the power
+                                if constexpr (kCap) {
+                                    ox = nq.x < -kAlphaCap;
+                                    oy = nq.y < -kAlphaCap;
+                                    nq = make_float2(fmaxf(nq.x, -kAlphaCap), fmaxf(nq.y, -kAlphaCap));
+                                }
+                                const float2 om = add2(one2, nq);
+                                // (rcp.approx(1) = 1: a pixel that does not blend keeps its T)
+                                const float2 inv = make_float2(rcp_approx(om.x), rcp_approx(om.y));
+                                const float2 Ti = mul2(T[q], inv);
+                                const float2 nw = mul2(nq, Ti);
+                                float2 nX;
+                                if constexpr (kAux) {
+                                    nX = add2(fma2(nC2[q], b2, fma2(nC1[q], g2, mul2(nC0[q], r2))), fma2(nD[q], z2, nO[q]));
+                                    zv = q ? fma2(nD[q], nw, zv) : mul2(nD[q], nw);
+                                } else {
+                                    nX = fma2(nC2[q], b2, fma2(nC1[q], g2, mul2(nC0[q], r2)));
+                                }
+                                // -dL/dalpha, then dL/dpower = dL/dalpha alpha
+                                float2 gp = mul2(fma2(Ti, nX, mul2(inv, S[q])), nq);
+                                if constexpr (kCap) gp = make_float2(ox ? 0.f : gp.x, oy ? 0.f : gp.y);
+                                S[q] = fma2(nX, nw, S[q]);
+                                T[q] = Ti;
+                                const float2 my = mul2(gp, dy[u][q]);
+                                c0v = q ? fma2(nC0[q], nw, c0v) : mul2(nC0[q], nw);
+                                c1v = q ? fma2(nC1[q], nw, c1v) : mul2(nC1[q], nw);
+                                c2v = q ? fma2(nC2[q], nw, c2v) : mul2(nC2[q], nw);
+                                A0v = q ? add2(A0v, gp) : gp;
+                                M1v = q ? add2(M1v, my) : my;
+                                M2v = q ? fma2(my, dy[u][q], M2v) : mul2(my, dy[u][q]);
+                            }
+                        };
+                        if (pf[u] & kCappedEntry) pairs(std::true_type{});
+                        else pairs(std::false_type{});
+                        A0 = A0v.x + A0v.y; M1 = M1v.x + M1v.y; M2 = M2v.x + M2v.y;
+                        c0 = c0v.x + c0v.y; c1 = c1v.x + c1v.y; c2 = c2v.x + c2v.y;
+                        if constexpr (kAux) zs = zv.x + zv.y;
+                    } else {
+                        A0 = M1 = M2 = c0 = c1 = c2 = 0.f;
+                        auto one = [&](float nr, float dyp, float &t, float &Sp, float h0, float h1, float h2, float hd,
+                                       float ho) {
+                            if (!(nr < 0.f)) return;
+                            const float nal = fmaxf(nr, -kAlphaCap);
+                            const float inv = rcp_approx(1.0f + nal);
+                            const float Ti = t * inv, nw = nal * Ti;
+                            float nX = h0 * r2.x + h1 * g2.x + h2 * b2.x;
+                            if constexpr (kAux) {
+                                nX += hd * z2.x + ho;
+                                zs += hd * nw;
+                            }
+                            c0 += h0 * nw;
+                            c1 += h1 * nw;
+                            c2 += h2 * nw;
+                            if (nr >= -kAlphaCap) {
+                                const float gp = (inv * Sp + Ti * nX) * nal, my = gp * dyp;
+                                A0 += gp;
+                                M1 += my;
+                                M2 += my * dyp;
+                            }
+                            Sp += nX * nw;
+                            t = Ti;
+                        };
+#pragma unroll
+                        for (int q = 0; q < NP; q++) {
+                            one(na[u][q].x, dy[u][q].x, T[q].x, S[q].x, nC0[q].x, nC1[q].x, nC2[q].x, nD[q].x, nO[q].x);
+                            one(na[u][q].y, dy[u][q].y, T[q].y, S[q].y, nC0[q].y, nC1[q].y, nC2[q].y, nD[q].y, nO[q].y);
+                        }
+                    }
+                    // the pixels share dx: m_x = dx m_0, m_xx = dx m_x, m_xy = dx m_y
+                    const float mx = dx[u] * A0;
+                    buf.h[k0 + u][0][lane] = make_float4(dx[u] * mx, dx[u] * M1, M2, A0);
+                    buf.h[k0 + u][1][lane] = make_float4(mx, M1, c0, c1);
+                    buf.e[0][k0 + u][lane] = c2;
+                    if constexpr (kAux) buf.e[1][k0 + u][lane] = zs;
+                }
+                valid |= any << k0;
             }
+            if (valid) flush_terms<NT>(buf, Sg, base, valid, lane, P);
         }
-        __syncthreads();
-        for (int k = tid; k < cnt; k += BLOCK)
-            flush_entry(&P.g2d[10 * (size_t)s_m[k]], &s_acc[k * NG], s0[k].z, s0[k].w, s1[k].x, s2[k].x, s2[k].y,
-                        s2[k].z);
-        end = start;
+        __syncwarp();  // the next group restages
     }
-}
-
-template <int TW, int TH, int PX>
-void launch_bwd_t(const Params &p, cudaStream_t s) {
-    note_launch();
-    if (p.aux)
-        pdl_launch(k_composite_bwd<TW, TH, PX, true>, p.total_tiles, TW * TH / PX, 0, s, p);
-    else
-        pdl_launch(k_composite_bwd<TW, TH, PX, false>, p.total_tiles, TW * TH / PX, 0, s, p);
 }
 
 }  // namespace
 
-#define PVG_DISPATCH_ONE_bwd(W, H, X) \
-    if (p.tile_w == W && p.tile_h == H && p.px == X) return launch_bwd_t<W, H, X>(p, s);
-
 void launch_composite_bwd(const Params &p, cudaStream_t s) {
     if (p.total_tiles == 0) return;
-    PVG_TILE_CONFIGS(PVG_DISPATCH_ONE_bwd)
+    const WarpShape w = warp_shape(p, kBwdWide4, kBwdWide8);
+    Params q = p;
+    q.block_shift = w.shift;
+    q.blocks_per_tile = w.blocks;
+    const uint32_t grid = p.total_tiles * w.blocks;
+    note_launch();
+    if (w.px == 8) {
+        if (p.aux) pdl_launch(k_composite_bwd<8, true>, grid, 32, 0, s, q);
+        else pdl_launch(k_composite_bwd<8, false>, grid, 32, 0, s, q);
+    } else if (w.px == 4) {
+        if (p.aux) pdl_launch(k_composite_bwd<4, true>, grid, 32, 0, s, q);
+        else pdl_launch(k_composite_bwd<4, false>, grid, 32, 0, s, q);
+    } else {
+        if (p.aux) pdl_launch(k_composite_bwd<2, true>, grid, 32, 0, s, q);
+        else pdl_launch(k_composite_bwd<2, false>, grid, 32, 0, s, q);
+    }
 }
 
 }  // namespace pvg

@@ -1,46 +1,163 @@
-// raster_common.cuh -- tile geometry and record staging shared by the
+// raster_common.cuh -- the warp's walk over its tile's list, shared by the
 // compositor (raster.cu) and its adjoint (raster_bwd.cu).
+//
+// One warp per CTA owns a block of 32 PX pixels of a tile: lanes in 8
+// columns x 4 rows (16 x 2 for tiles of 8 rows with PX = 4, and for PX = 8),
+// each lane PX vertically adjacent pixels.  It takes the tile's sorted list 32 entries at
+// a time, one per lane: the lane tests whether the entry's footprint can
+// reach the block at all (block_hit) and the hits are compacted into shared
+// memory, so that the loop over entries only sees those.  No warp waits for
+// another: a block whose pixels have all stopped ends at once, the blocks of
+// a long list run on different SMs, and no barrier separates the batches.
 #pragma once
 #include "pvg_internal.cuh"
 
 namespace pvg {
 namespace {
 
-struct TileGeom {
+struct BlockGeom {
     const ViewDesc *V;
-    int px, py0;  // this thread's first pixel (column px, rows py0 .. py0 + PX - 1)
-    uint2 r;      // list range
+    uint32_t tile;
+    int px, py0;          // this lane's first pixel (column px, rows py0 .. py0 + PX - 1)
+    float x0, x1, y0, y1; // centres of the block's outermost pixels
+    uint2 r;              // list range
 };
 
-template <int TW, int TH, int PX>
-__device__ __forceinline__ TileGeom tile_geom(const Params &P) {
-    static_assert(TW % 8 == 0 && (TH / PX) % 4 == 0 && TH % PX == 0, "tile must be whole 8x4-thread warps");
-    TileGeom g;
-    const uint32_t tile = P.tile_order ? P.tile_order[blockIdx.x] : blockIdx.x;
-    const int view = view_of_tile(P.views, P.n_views, tile);
-    g.V = &P.views[view];
-    const uint32_t lt = tile - g.V->tile_base;
-    const int tx = (int)(lt % (uint32_t)g.V->tiles_x), ty = (int)(lt / (uint32_t)g.V->tiles_x);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wx = warp % (TW / 8), wy = warp / (TW / 8);
-    g.px = tx * TW + wx * 8 + (lane & 7);
-    g.py0 = ty * TH + (wy * 4 + (lane >> 3)) * PX;
-    g.r = P.ranges[tile];
+template <int PX>
+__device__ __forceinline__ BlockGeom block_geom(const Params &P) {
+    BlockGeom g;
+    const uint32_t t = blockIdx.x / P.blocks_per_tile, sub = blockIdx.x % P.blocks_per_tile;
+    g.tile = P.tile_order ? P.tile_order[t] : t;
+    g.V = &P.views[view_of_tile(P.views, P.n_views, g.tile)];
+    const uint32_t lt = g.tile - g.V->tile_base;
+    const int bw = 1 << P.block_shift, bh = (32 >> P.block_shift) * PX;
+    const uint32_t nbx = (uint32_t)P.tile_w >> P.block_shift;
+    const int bx = (int)(lt % (uint32_t)g.V->tiles_x) * P.tile_w + (int)(sub % nbx) * bw;
+    const int by = (int)(lt / (uint32_t)g.V->tiles_x) * P.tile_h + (int)(sub / nbx) * bh;
+    const int lane = threadIdx.x;
+    g.px = bx + (lane & (bw - 1));
+    g.py0 = by + (lane >> P.block_shift) * PX;
+    g.x0 = (float)bx + 0.5f;
+    g.x1 = (float)(bx + bw) - 0.5f;
+    g.y0 = (float)by + 0.5f;
+    g.y1 = (float)(by + bh) - 0.5f;
+    g.r = P.ranges[g.tile];
     return g;
 }
 
-__device__ __forceinline__ void stage_record(const Params &P, uint32_t m, float4 *s0, float2 *s1, float4 *s2,
-                                             int slot) {
-    float4 a, c;
-    float2 b;
-    record_terms(P.rec, m, a, b, c);
-    s0[slot] = a;
-    s1[slot] = b;
-    s2[slot] = c;
+// Whether an entry can blend at a pixel centre of [x0, x1] x [y0, y1]:
+// false only when the largest exponent a' dx^2 + b' dx dy + c' dy^2 over the
+// rectangle is below -log2(255 o~), so that alpha < 1/255 everywhere on it.
+// The form is concave: its maximum over a rectangle that does not hold the
+// centre lies on the edge nearest in x or the one nearest in y, at that
+// edge's own maximum clamped into it.  The level is widened by 1 % + 1e-4
+// against the rounding of the compositor's own evaluation, and needle
+// footprints ((a + c)^2 > 1e4 (ac - b^2), where that rounding may exceed it)
+// and non-finite entries always count as hits, so culling changes no image.
+__device__ __forceinline__ bool block_hit(float u, float v, float ap, float bp, float cp, float ot, float x0,
+                                          float x1, float y0, float y1) {
+    const float hb = 0.5f * bp, tr = ap + cp;
+    const bool well = tr * tr <= 1e4f * diff_of_products(ap, cp, hb, hb);
+    const float level = -(1.01f * fmaxf(lg2_approx(255.0f * ot), 0.0f) + 1e-4f);
+    const float ax = x0 - u, bx = x1 - u, ay = y0 - v, by = y1 - v;
+    const float xe = fminf(fmaxf(0.0f, ax), bx), ye = fminf(fmaxf(0.0f, ay), by);
+    const float ys = fminf(fmaxf(-hb * xe * rcp_approx(cp), ay), by);
+    const float xs = fminf(fmaxf(-hb * ye * rcp_approx(ap), ax), bx);
+    const float p1 = ap * xe * xe + ys * (bp * xe + cp * ys), p2 = cp * ye * ye + xs * (bp * ye + ap * xs);
+    return !(well && p1 < level && p2 < level);
 }
 
+// flags beside an entry's list position
+constexpr uint32_t kOddEntry = 0x80000000u;     // non-finite terms: pixels one at a time
+constexpr uint32_t kCappedEntry = 0x40000000u;  // o~ may exceed the alpha cap
+constexpr uint32_t kPosMask = 0x3fffffffu;      // a list of 2^30 entries does not fit the device memory
+
+constexpr int kStagedPlaces = 32;
+
+// The hits of 32 list entries, operands of the packed arithmetic in pairs.
+struct Staged {
+    float4 a[kStagedPlaces];  // (u, a', b', list position | flags)
+    float4 b[kStagedPlaces];  // (v, v, c', c')
+    float4 c[kStagedPlaces];  // (-o~, -o~, r, r)
+    float4 d[kStagedPlaces];  // (g, g, b, b)
+    float2 e[kStagedPlaces];  // (z, z)
+    uint32_t m[kStagedPlaces];
+};
+
+// 32 records on their way to shared memory, one per lane
+struct RawRecords {
+    float4 q[3][32];
+};
+
+constexpr uint32_t kNoRecord = 0xffffffffu;
+
+// starts the copy of record m into the lane's place
+__device__ __forceinline__ void fetch_record(const Params &P, RawRecords &raw, uint32_t m, int lane) {
+    if (m == kNoRecord) return;
+    const float4 *src = P.rec + 3 * (size_t)m;
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(&raw.q[k][lane])),
+                     "l"(src + k)
+                     : "memory");
+}
+
+__device__ __forceinline__ void wait_records() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The lane's record (arrived), tested and, if it can reach the block,
+// written to the next free place of S; returns the number of hits.  pos: the
+// record's list position.  The places up to the next multiple of U get an
+// entry that blends nowhere.
+template <int U>
+__device__ __forceinline__ int stage_hits(const RawRecords &raw, Staged &S, bool have, uint32_t m, uint32_t pos,
+                                          const BlockGeom &G, int lane) {
+    bool hit = false;
+    float4 a, c;
+    float2 b;
+    if (have) {
+        const float4 q[3] = {raw.q[0][lane], raw.q[1][lane], raw.q[2][lane]};
+        record_terms(q, 0, a, b, c);
+        hit = block_hit(a.x, a.y, a.z, a.w, b.x, b.y, G.x0, G.x1, G.y0, G.y1);
+    }
+    const uint32_t mask = __ballot_sync(0xffffffffu, hit);
+    if (hit) {
+        const int k = __popc(mask & ((1u << lane) - 1u));
+        // finite: no term is NaN or infinite, so that 0 weights keep sums unchanged
+        const float s = fabsf(a.x) + fabsf(a.y) + fabsf(a.z) + fabsf(a.w) + fabsf(b.x) + fabsf(b.y) + fabsf(c.x) +
+                        fabsf(c.y) + fabsf(c.z) + fabsf(c.w);
+        pos |= (s < 1e30f ? 0u : kOddEntry) | (b.y <= kUncappedOpacity ? 0u : kCappedEntry);
+        S.a[k] = make_float4(a.x, a.z, a.w, __uint_as_float(pos));
+        S.b[k] = make_float4(a.y, a.y, b.x, b.x);
+        S.c[k] = make_float4(-b.y, -b.y, c.x, c.x);
+        S.d[k] = make_float4(c.y, c.y, c.z, c.z);
+        S.e[k] = make_float2(c.w, c.w);
+        S.m[k] = m;
+    }
+    const int hits = __popc(mask);
+    if (U > 1 && lane < (U - hits % U) % U) {
+        const int k = hits + lane;
+        S.a[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        S.b[k] = make_float4(0.f, 0.f, -kMinRowCoef, -kMinRowCoef);
+        S.c[k] = S.d[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        S.e[k] = make_float2(0.f, 0.f);
+        S.m[k] = 0u;
+    }
+    __syncwarp();
+    return hits;
+}
 
 }  // namespace
+
+// Pixels per lane of the compositing kernels and the block's shape in a
+// tile.  A lane takes eight (four) pixels when the frame has wide8 blocks of
+// 256 (wide4 of 128) pixels per SM, else two.
+struct WarpShape {
+    int px, shift;
+    uint32_t blocks;  // per tile
+};
+WarpShape warp_shape(const Params &p, int wide4, int wide8);
+
 }  // namespace pvg
 
 // Supported (tile width, tile height, pixels per thread) combinations.

@@ -849,17 +849,19 @@ __device__ __forceinline__ void tile_order_block(const uint2 *__restrict__ range
 }
 
 __global__ void __launch_bounds__(1024) k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles,
-                                                     uint32_t *__restrict__ order) {
+                                                     uint32_t *__restrict__ order, uint32_t *__restrict__ walk) {
     pdl_enter();
+    if (walk)
+        for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x) walk[t] = 0u;
     tile_order_block(ranges, nullptr, n_tiles, order);
 }
 
-// The adjoint's first kernel: rows [0, *d_m) of a [*, per] array zeroed
-// (the visible items' image-space gradients, which the adjoint accumulates)
-// by all blocks but the last, which orders the tiles by their walk lengths
-// and resets the per-item adjoint's chunk ticket (counters[3]).
-__global__ void __launch_bounds__(1024) k_bwd_prep(float *__restrict__ a, const uint32_t *d_m, int per,
-                                                  const uint32_t *walk, uint32_t n_tiles,
+// The adjoint's first kernel: rows [0, *d_m) of the image-space gradients
+// zeroed (the visible items', which the adjoint accumulates) by all blocks
+// but the last, which orders the tiles by their walk lengths and resets the
+// per-item adjoint's chunk ticket (counters[3]).
+__global__ void __launch_bounds__(1024) k_bwd_prep(double *__restrict__ g2m, float *__restrict__ g2d,
+                                                  const uint32_t *d_m, const uint32_t *walk, uint32_t n_tiles,
                                                   uint32_t *__restrict__ order, uint32_t *ticket) {
     pdl_enter();
     if (blockIdx.x == gridDim.x - 1) {
@@ -867,20 +869,22 @@ __global__ void __launch_bounds__(1024) k_bwd_prep(float *__restrict__ a, const 
         tile_order_block(nullptr, walk, n_tiles, order);
         return;
     }
-    const size_t n = (size_t)per * *d_m;
-    const size_t stride = (size_t)(gridDim.x - 1) * blockDim.x;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += stride) a[k] = 0.f;
+    const size_t M = *d_m, stride = (size_t)(gridDim.x - 1) * blockDim.x;
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    for (size_t k = first; k < 3 * M; k += stride) g2m[k] = 0.0;
+    float4 *rows = reinterpret_cast<float4 *>(g2d);
+    for (size_t k = first; k < kG2dRow / 4 * M; k += stride) rows[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 void launch_tile_order(const Params &p, cudaStream_t s) {
     if (p.total_tiles == 0) return;
     note_launch();
-    pdl_launch(k_tile_order, 1, 1024, 0, s, p.ranges, p.total_tiles, p.tile_order);
+    pdl_launch(k_tile_order, 1, 1024, 0, s, p.ranges, p.total_tiles, p.tile_order, p.tile_walk);
 }
 
 void launch_bwd_prep(const Params &p, const uint32_t *walk, uint32_t *order, cudaStream_t s) {
     note_launch();
-    pdl_launch(k_bwd_prep, device_sm_count() + 1, 1024, 0, s, p.g2d, (const uint32_t *)&p.counters[0], 10, walk,
+    pdl_launch(k_bwd_prep, device_sm_count() + 1, 1024, 0, s, p.g2m, p.g2d, (const uint32_t *)&p.counters[0], walk,
                p.total_tiles, order, &p.counters[3]);
 }
 
