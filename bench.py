@@ -241,7 +241,8 @@ def parse_clock_lines(lines):
 
 
 # the sources that decide the compositor kernels' memory traffic
-COMPOSITOR_SOURCES = ("pvg_internal.cuh", "raster_common.cuh", "raster.cu", "raster_bwd.cu")
+COMPOSITOR_SOURCES = ("pvg_internal.cuh", "raster_common.cuh", "raster_fwd.cuh", "raster.cu", "raster_bwd.cuh",
+                      "raster_bwd.cu")
 
 
 def kernel_source_hash(files=COMPOSITOR_SOURCES):

@@ -716,8 +716,7 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
     f->pair_capacity = pair_cap;
     p.pair_vals = ptr<uint32_t>(f->pair_vals);
     tm.begin(PVG_STAGE_COMPOSITE, s);
-    launch_composite(p, s);
-    if (n_feat) launch_composite_feat(p, s);
+    launch_composite(p, s);  // with the extra channels, if any
     tm.end(PVG_STAGE_COMPOSITE, s);
     tm.on = timer_on;
     PVG_CUDA(cudaGetLastError());
@@ -938,12 +937,11 @@ extern "C" pvg_status_t pvg_render_bwd(pvg_ctx_t *x, const pvg_scene_t *scene, c
     // forward recorded each tile's largest last-blend position)
     launch_bwd_prep(p, ptr<uint32_t>(f->tile_walk), ptr<uint32_t>(f->tile_order_bwd), s);
     p.tile_order = ptr<uint32_t>(f->tile_order_bwd);
-    launch_composite_bwd(p, s);
     if (feat_bwd && f->n_items) {
         note_launch();
         pdl_launch(k_zero_rows, device_sm_count() * 4, 256, 0, s, p.gfeat, &p.counters[0], p.n_feat);
-        launch_composite_feat_bwd(p, s);
     }
+    launch_composite_bwd(p, s);  // with the extra channels' adjoint, if any
     tm.end(PVG_STAGE_COMPOSITE_BWD, s);
     tm.begin(PVG_STAGE_PREPROCESS_BWD, s);
     launch_preprocess_bwd(p, n_views > 1, s);

@@ -109,9 +109,11 @@ __device__ __forceinline__ void wait_records() { asm volatile("cp.async.wait_all
 // written to the next free place of S; returns the number of hits.  pos: the
 // record's list position.  The places up to the next multiple of U get an
 // entry that blends nowhere.
+// items (optional): the hits' values of `item`, in their places.
 template <int U>
 __device__ __forceinline__ int stage_hits(const RawRecords &raw, Staged &S, bool have, uint32_t m, uint32_t pos,
-                                          const BlockGeom &G, int lane) {
+                                          const BlockGeom &G, int lane, uint32_t item = 0,
+                                          uint32_t *items = nullptr) {
     bool hit = false;
     float4 a, c;
     float2 b;
@@ -133,6 +135,7 @@ __device__ __forceinline__ int stage_hits(const RawRecords &raw, Staged &S, bool
         S.d[k] = make_float4(c.y, c.y, c.z, c.z);
         S.e[k] = make_float2(c.w, c.w);
         S.m[k] = m;
+        if (items) items[k] = item;
     }
     const int hits = __popc(mask);
     if (U > 1 && lane < (U - hits % U) % U) {
@@ -145,6 +148,78 @@ __device__ __forceinline__ int stage_hits(const RawRecords &raw, Staged &S, bool
     }
     __syncwarp();
     return hits;
+}
+
+// Extra channels of the staged entries, each value twice (operands of the
+// packed arithmetic), zeros beyond the call's channels.
+template <int NG>
+struct StagedFeats {
+    alignas(16) float2 f[kStagedPlaces][4 * NG];
+    uint32_t item[kStagedPlaces];  // Gaussian of the entry's scene
+};
+template <>
+struct StagedFeats<0> {};
+
+// Zeroes the channel values once: those beyond the call's channels stay zero.
+template <int NG>
+__device__ __forceinline__ void clear_feats(StagedFeats<NG> &F, int lane) {
+    for (int k = lane; k < kStagedPlaces * 2 * NG; k += 32)
+        reinterpret_cast<float4 *>(&F.f[0][0])[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// The channel values of the `hits` staged entries (their Gaussians in
+// F.item; places up to the next multiple of U zeroed): every semantic row by
+// the whole warp, all rows' copies in flight together and behind them v_bar
+// and rho by the entries' lanes; then one pass doubles the semantic values.
+// Entries with non-finite values are flagged in S.
+template <int NG, int U>
+__device__ __forceinline__ void stage_feats(const Params &P, const ViewDesc &V, Staged &S, StagedFeats<NG> &F,
+                                            int hits, int lane) {
+    const int places = (hits + U - 1) / U * U;
+    const int c0 = ((P.feat_mask & kFeatVbar) ? 3 : 0) + ((P.feat_mask & kFeatRho) ? 1 : 0);
+    const int n_sem = (P.feat_mask & kFeatSem) ? V.n_sem : 0;
+    if (lane < n_sem) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&F.f[0][c0 + lane].x);
+        for (int k = 0; k < hits; k++)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + k * (uint32_t)sizeof(F.f[0])),
+                         "l"(V.sem + (size_t)F.item[k] * n_sem + lane)
+                         : "memory");
+    }
+    if (c0 && lane < hits) {
+        const uint32_t i = F.item[lane];
+        const float rho = __fdiv_rn(V.beta[i], V.period[i]);
+        float bad = 0.f;
+        int c = 0;
+        auto put = [&](float v) {
+            F.f[lane][c++] = make_float2(v, v);
+            bad += fabsf(v);
+        };
+        if (P.feat_mask & kFeatVbar) {
+            const float w = expf(-0.5f * rho);
+            const float3 vel = make_float3(V.vel[3 * (size_t)i], V.vel[3 * (size_t)i + 1], V.vel[3 * (size_t)i + 2]);
+            put(vel.x * w);
+            put(vel.y * w);
+            put(vel.z * w);
+        }
+        if (P.feat_mask & kFeatRho) put(fminf(rho, 2.0f));
+        if (!(bad < 1e30f)) S.a[lane].w = __uint_as_float(__float_as_uint(S.a[lane].w) | kOddEntry);
+    }
+    for (int k = hits; k < places; k++)
+        for (int c = lane; c < 4 * NG; c += 32) F.f[k][c] = make_float2(0.f, 0.f);
+    if (n_sem) {
+        wait_records();
+        uint32_t bad = 0;  // entries with a non-finite value of this lane's class
+        if (lane < n_sem)
+#pragma unroll 4
+            for (int k = 0; k < hits; k++) {
+                const float v = F.f[k][c0 + lane].x;
+                F.f[k][c0 + lane].y = v;
+                bad |= fabsf(v) < 1e30f ? 0u : 1u << k;
+            }
+        bad = __reduce_or_sync(0xffffffffu, bad);
+        if ((bad >> lane) & 1u) S.a[lane].w = __uint_as_float(__float_as_uint(S.a[lane].w) | kOddEntry);
+    }
+    __syncwarp();
 }
 
 }  // namespace

@@ -96,3 +96,37 @@ def test_non_finite_values_stay_where_they_blend(cfg, repeat):
     grads = r.backward(st, cams, fr, [d] * len(cams))
     assert 0 < int(blended.sum()) < 200
     assert torch.equal(~torch.isfinite(grads["opacity"]), blended)
+
+
+@pytest.mark.parametrize("mask,n_sem", [(abi.FEAT_RHO, 0), (abi.FEAT_VBAR, 0), (abi.FEAT_SEM, 1), (abi.FEAT_SEM, 32),
+                                        (abi.FEAT_VBAR | abi.FEAT_SEM, 30), (7, 19), (7, 32)])
+def test_channels_keep_the_colour_pass_and_their_non_finite_values(mask, n_sem):
+    """Colour, depth and opacity rendered with channels equal the plain
+    render's bit for bit and their gradients agree (one view, equal sums in
+    another order: 1e-4 of the norm); a class value that is not finite shows
+    exactly where its Gaussian has a weight."""
+    scene = synth.make_plain_scene(seed=9, n=200, log_scale_mean=-2.3)
+    st = R.scene_to_device(scene)
+    cam = synth.plain_camera(75, 53, t=0.5)
+    r, fr, fp = R.Renderer(), R.Frame(), R.Frame()
+    plain = r.forward(st, [cam], frame=fp)[0]
+    if n_sem:
+        st["sem"] = torch.tensor(synth.make_semantics(200, n_sem), device="cuda")
+    out = r.forward(st, [cam], frame=fr, features=mask)[0]
+    for k in ("rgb", "depth", "alpha"):
+        assert torch.equal(out[k], plain[k]), k
+    d = _weights(cam, True)
+    want = r.backward(st, [cam], fp, [d])
+    got = r.backward(st, [cam], fr, [dict(d, feat=torch.zeros_like(out["feat"]))])
+    for k in R.PARAM_NAMES:
+        assert torch.linalg.norm(got[k] - want[k]) <= 1e-4 * torch.linalg.norm(want[k]), k
+    if n_sem:
+        who = int(np.argmax(scene["opacity"]))
+        st["sem"] = torch.zeros(200, n_sem, device="cuda")
+        st["sem"][who, n_sem - 1] = 1.0
+        weight = r.forward(st, [cam], features=mask)[0]["feat"][-1]
+        st["sem"][who, n_sem - 1] = float("nan")
+        feat = r.forward(st, [cam], features=mask)[0]["feat"]
+        assert 0 < int((weight > 0).sum()) < weight.numel()
+        assert torch.equal(torch.isnan(feat[-1]), weight > 0)
+        assert torch.isfinite(feat[:-1]).all()
