@@ -107,9 +107,12 @@ class Renderer:
         abi.check(self._lib.pvg_create(C.byref(h), C.byref(self.cfg)), "pvg_create")
         self.handle = h
         self.device = torch.cuda.current_device()
+        self._frames = []  # (stream, frame): idle frames of render_differentiable
 
     def close(self):
         if self.handle:
+            while self._frames:
+                self._frames.pop()[1].close()
             self._lib.pvg_destroy(self.handle)
             self.handle = None
 
@@ -247,6 +250,57 @@ def render(scene_t, cams, renderer=None, frame=None, features=0):
     return r.forward(scene_t, cams, frame=frame, features=features)
 
 
+class _FrameLease:
+    """The frame of one differentiable render, from its renderer's idle
+    frames or new, and given back by ``release`` (or when dropped).  A frame
+    holds some 20 device buffers, and creating and freeing them was most of a
+    small differentiable render.  An idle frame is only lent to the stream
+    that used it last, behind whose work it is free.  A renderer keeps at
+    most ``KEEP`` idle frames and frees them with itself; a lease taken while
+    the stream is being captured is a frame of its own."""
+
+    KEEP = 4
+
+    def __init__(self, renderer):
+        self.renderer = renderer
+        self.frame = None
+        self.stream = torch.cuda.current_stream().cuda_stream
+        self.own = torch.cuda.is_current_stream_capturing()
+        if not self.own:
+            for _ in range(len(renderer._frames)):
+                try:
+                    stream, frame = renderer._frames.pop()
+                except IndexError:  # another thread's
+                    break
+                if stream == self.stream:
+                    self.frame = frame
+                    break
+                renderer._frames.insert(0, (stream, frame))
+        if self.frame is None:
+            self.frame = Frame()
+
+    @property
+    def handle(self):
+        return self.frame.handle if self.frame is not None else None
+
+    def release(self, stream=None):
+        """``stream``: the last call's, if it was not the lease's."""
+        frame, self.frame = self.frame, None
+        if frame is None:
+            return
+        r = self.renderer
+        if self.own or r.handle is None or stream not in (None, self.stream) or len(r._frames) >= self.KEEP:
+            frame.close()
+        else:
+            r._frames.append((self.stream, frame))
+
+    def __del__(self):
+        try:
+            self.release()
+        except Exception:
+            pass
+
+
 class PVGRender(torch.autograd.Function):
     """images = Render({H_i(t)}; E, I) (Sec. 3.2, Eq. 8) for one camera,
     differentiable w.r.t. all nine parameter arrays and the optional sky
@@ -259,7 +313,7 @@ class PVGRender(torch.autograd.Function):
                        opacity=opacity.contiguous(), sh=sh.contiguous())
         if sky is not None:
             scene_t["sky"] = sky.contiguous()
-        frame = Frame()
+        frame = _FrameLease(renderer)
         out = renderer.forward(scene_t, [cam], frame=frame)[0]
         ctx.cam, ctx.renderer, ctx.frame = cam, renderer, frame
         ctx.has_sky = sky is not None
@@ -274,7 +328,7 @@ class PVGRender(torch.autograd.Function):
             scene_t["sky"] = saved[len(PARAM_NAMES)]
         grads = ctx.renderer.backward(scene_t, [ctx.cam], ctx.frame,
                                       [dict(rgb=g_rgb, depth=g_depth, alpha=g_alpha)])
-        ctx.frame.close()
+        ctx.frame.release(torch.cuda.current_stream().cuda_stream)
         return (None, None) + tuple(grads[k] for k in PARAM_NAMES) + (grads.get("sky"),)
 
 
