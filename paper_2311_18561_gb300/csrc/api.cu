@@ -635,6 +635,8 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
     p.pix_last = ptr<uint32_t>(f->pix_last);
     p.pix_neval = ptr<uint32_t>(f->pix_neval);
     p.vis_off = ptr<uint32_t>(x->vis_off);
+    p.vis_tile = p.item_zkey;  // both dead after the compaction
+    p.vis_stride = p.item_cnt;
     p.feat_mask = fmask;
     p.n_feat = n_feat;
     if (!keep_state) p.pix_T = nullptr;  // inference only: no state for a backward pass

@@ -72,6 +72,10 @@ __global__ void __launch_bounds__(256, 4) k_finalize(Params P) {
         F.mut = make_float3(q2.x, q2.y, q2.z);
         const uint32_t r0 = __float_as_uint(q2.w), r1 = __float_as_uint(q3.x);
         F.tx0 = r0 & 0xffffu; F.ty0 = r0 >> 16; F.tx1 = r1 & 0xffffu; F.ty1 = r1 >> 16;
+        if (P.n_views > 1) {  // the expansion's tile ids without a search for the view
+            P.vis_tile[m] = V.tile_base + F.ty0 * (uint32_t)V.tiles_x + F.tx0;
+            P.vis_stride[m] = (uint32_t)V.tiles_x;
+        }
         float dx = F.mut.x - V.campos[0], dy = F.mut.y - V.campos[1], dz = F.mut.z - V.campos[2];
         const float inv = 1.0f / sqrtf(dx * dx + dy * dy + dz * dz);
         dx *= inv; dy *= inv; dz *= inv;

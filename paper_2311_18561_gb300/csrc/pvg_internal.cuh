@@ -107,6 +107,9 @@ struct Params {
     uint2 *rect;             // [M]
     uint32_t *vis_cnt;       // [M] tiles per visible item
     uint32_t *vis_off;       // [M] first pair position of the item
+    uint32_t *vis_tile;      // [M] several views: id of the rectangle's first tile (in item_zkey's space,
+                             // dead after the compaction)
+    uint32_t *vis_stride;    // [M] several views: tiles per row of the view (in item_cnt's space)
     uint32_t *chunk_start;   // [K / 2048 + 1] first item of each pair chunk
     // pairs
     uint32_t *pair_keys;     // [K] tile ids (sorted in place via ping-pong)

@@ -24,6 +24,8 @@
 // bit (the lanes holding the same digit, then those before it).  The first
 // digit pass's histogram can be counted by the kernel that writes the keys
 // (compaction, pair expansion), which saves that pass's upsweep.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <atomic>
 #include "pvg_internal.cuh"
@@ -331,19 +333,24 @@ __global__ void __launch_bounds__(1024) k_radix_scan(uint32_t *hist, uint32_t *t
 // first output falls in the chunk marks that slot with its m; the scan
 // carries the last mark forward).  Its r-th pair is the r-th tile, row by
 // row, of the rectangle tiles that its footprint ellipse meets: read from
-// the item's packed row table when it has one (at most kTabRows rows),
-// else recomputed from the stored ellipse, 32 rows at a time by the whole
-// warp, for one such item after another.  The kernel also counts the
-// first digit pass of the tile sort that follows (hist, zeroed by the
-// scan before it): each chunk's outputs are contiguous, so their counts
-// are summed in shared memory per sort block and added with atomics.
-__global__ void __launch_bounds__(kEmitThreads) k_expand_pairs(const uint32_t *__restrict__ vis_off,
+// the item's packed row table when it has one (at most kTabRows rows).  The
+// chunk's items without a table are listed and taken one after another by
+// whole warps, which evaluate 32 rows of the stored ellipse at once and then
+// write all of the item's outputs in those rows (evaluating the rows for
+// every 32 outputs made the batched views' expansion 292 M warp instructions
+// for 40 M pairs).  The kernel also counts the first digit pass of the tile
+// sort that follows (hist, zeroed by the scan before it; NULL: none): each
+// chunk's outputs are contiguous, so their counts are summed in shared
+// memory per sort block and added with atomics.
+template <uint32_t kEmitChunk>
+__global__ void __launch_bounds__(kEmitThreads, 4) k_expand_pairs(const uint32_t *__restrict__ vis_off,
                                                               const uint32_t *__restrict__ vis_cnt,
                                                               const uint32_t *__restrict__ chunk_start,
                                                               const uint2 *__restrict__ rect,
                                                               const uint4 *__restrict__ rowtab,
                                                               const float4 *__restrict__ ell, int tile_w,
-                                                              int tile_h, const uint32_t *__restrict__ sgid,
+                                                              int tile_h, const uint32_t *__restrict__ vis_tile,
+                                                              const uint32_t *__restrict__ vis_stride,
                                                               const ViewDesc *views, int nv, const uint32_t *d_m,
                                                               const uint32_t *d_k, uint32_t capacity,
                                                               uint32_t *__restrict__ keys, uint32_t *__restrict__ vals,
@@ -352,6 +359,8 @@ __global__ void __launch_bounds__(kEmitThreads) k_expand_pairs(const uint32_t *_
     pdl_enter();
     constexpr int kPer = kEmitChunk / kEmitThreads;  // slots per thread in the scan
     __shared__ uint32_t s_item[kEmitChunk];
+    __shared__ uint32_t s_big[kEmitChunk];  // the chunk's items without a table
+    __shared__ uint32_t s_nbig;
     __shared__ uint32_t s_warp[kEmitThreads / 32];
     __shared__ uint32_t s_hist[kCompactSpan][kRadix];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -367,8 +376,9 @@ __global__ void __launch_bounds__(kEmitThreads) k_expand_pairs(const uint32_t *_
         // sort blocks of the chunk's outputs: sb0 .. sb0 + nsb - 1 counted in
         // shared memory (any beyond kCompactSpan straight into hist)
         const uint32_t sb0 = j0 / seg;
-        const int nsb = (int)min((min(j0 + kEmitChunk, K) - 1) / seg - sb0 + 1, (uint32_t)kCompactSpan);
+        const int nsb = !hist ? 0 : (int)min((min(j0 + kEmitChunk, K) - 1) / seg - sb0 + 1, (uint32_t)kCompactSpan);
         __syncthreads();
+        if (threadIdx.x == 0) s_nbig = 0u;
         for (int q = threadIdx.x; q < (int)kEmitChunk; q += kEmitThreads) s_item[q] = 0u;
         for (int q = threadIdx.x; q < nsb * kRadix; q += kEmitThreads) (&s_hist[0][0])[q] = 0u;
         __syncthreads();
@@ -378,7 +388,12 @@ __global__ void __launch_bounds__(kEmitThreads) k_expand_pairs(const uint32_t *_
         if (threadIdx.x == 0) s_item[0] = m_lo;
         for (uint32_t m = m_lo + threadIdx.x; m <= m_hi; m += kEmitThreads) {
             const uint32_t o = vis_off[m];
-            if (o >= j0 && o - j0 < kEmitChunk && vis_cnt[m] > 0u) s_item[o - j0] = m;
+            const uint2 rc = rect[m];
+            const bool starts = o >= j0 && o - j0 < kEmitChunk && vis_cnt[m] > 0u;
+            if (starts) s_item[o - j0] = m;
+            if ((starts || m == m_lo) &&
+                !has_row_table(rc.x & 0xffffu, rc.x >> 16, rc.y & 0xffffu, rc.y >> 16))
+                s_big[atomicAdd(&s_nbig, 1u)] = m;
         }
         __syncthreads();
         // inclusive max-scan of the marks: kPer consecutive slots per
@@ -404,87 +419,102 @@ __global__ void __launch_bounds__(kEmitThreads) k_expand_pairs(const uint32_t *_
 #pragma unroll
         for (int i = 0; i < kPer; i++) s_item[threadIdx.x * kPer + i] = max(loc[i], before);
         __syncthreads();
-        // whole warps iterate together (kEmitChunk is a multiple of the
-        // block), so the warp-wide steps below see all 32 lanes
-        for (uint32_t q = threadIdx.x; q < kEmitChunk; q += kEmitThreads) {
-            const uint32_t j = j0 + q;
-            const bool valid = j < K;
-            if (!__any_sync(kFull, valid)) break;
-            const uint32_t m = valid ? s_item[q] : m_lo;
-            uint32_t r = valid ? j - vis_off[m] : 0u;
-            const uint2 rc = rect[m];
-            const uint32_t tx0 = rc.x & 0xffffu, ty0 = rc.x >> 16, tx1 = rc.y & 0xffffu, ty1 = rc.y >> 16;
-            uint32_t tx = tx0, ty = ty0;  // the rows sum to the item's count; first tile otherwise
-            const bool tab = has_row_table(tx0, ty0, tx1, ty1);
-            if (valid && tab) {
-                const uint4 t = rowtab[m];
-                const uint32_t w[4] = {t.x, t.y, t.z, t.w};
+        // output j of item m: its tile's id, and its digit counted
+        auto emit = [&](uint32_t j, uint32_t m, uint32_t key) {
+            keys[j] = key;
+            vals[j] = m;
+            if (!hist) return;
+            const uint32_t d = key & (kRadix - 1u), sb = j / seg - sb0;
+            if (sb < (uint32_t)nsb) atomicAdd(&s_hist[sb][d], 1u);
+            else atomicAdd(&hist[(size_t)d * sort_G + sb0 + sb], 1u);
+        };
+        const uint32_t tile0 = nv > 1 ? 0u : views[0].tile_base, stride0 = nv > 1 ? 0u : (uint32_t)views[0].tiles_x;
+        // items with a table, an output per thread; four outputs of a thread
+        // at a time, their items' data loaded together: the loads' latency
+        // bounds the expansion, not its bytes
+        constexpr int kAhead = kPer < 4 ? kPer : 4;
+        static_assert(kPer % kAhead == 0, "whole batches of outputs");
+        for (uint32_t q0 = threadIdx.x; q0 < kEmitChunk && j0 + q0 < K; q0 += kAhead * kEmitThreads) {
+            uint32_t am[kAhead], aoff[kAhead], atile[kAhead], astride[kAhead];
+            uint2 arc[kAhead];
+            uint4 atab[kAhead];
 #pragma unroll
-                for (int i = 0; i < (int)kTabRows; i++) {
-                    if (ty0 + i >= ty1) break;
-                    const uint32_t v = (w[i >> 1] >> (16 * (i & 1))) & 0xffffu;
+            for (int i = 0; i < kAhead; i++) am[i] = j0 + q0 + i * kEmitThreads < K ? s_item[q0 + i * kEmitThreads] : m_lo;
+#pragma unroll
+            for (int i = 0; i < kAhead; i++) {
+                aoff[i] = vis_off[am[i]];
+                arc[i] = rect[am[i]];
+                atab[i] = rowtab[am[i]];  // (not written for items without a table, and not used then)
+                atile[i] = nv > 1 ? vis_tile[am[i]] : 0u;
+                astride[i] = nv > 1 ? vis_stride[am[i]] : stride0;
+            }
+#pragma unroll
+            for (int i = 0; i < kAhead; i++) {
+                const uint32_t j = j0 + q0 + i * kEmitThreads;
+                const uint32_t tx0 = arc[i].x & 0xffffu, ty0 = arc[i].x >> 16, tx1 = arc[i].y & 0xffffu, ty1 = arc[i].y >> 16;
+                if (j >= K || !has_row_table(tx0, ty0, tx1, ty1)) continue;
+                const uint32_t w[4] = {atab[i].x, atab[i].y, atab[i].z, atab[i].w};
+                uint32_t r = j - aoff[i], col = 0, row = 0;  // the rows sum to the item's count
+#pragma unroll
+                for (int t = 0; t < (int)kTabRows; t++) {
+                    if (ty0 + t >= ty1) break;
+                    const uint32_t v = (w[t >> 1] >> (16 * (t & 1))) & 0xffffu;
                     const uint32_t sp = v >> 8;
                     if (r < sp) {
-                        tx = tx0 + (v & 0xffu) + r;
-                        ty = ty0 + i;
+                        col = (v & 0xffu) + r;
+                        row = t;
                         break;
                     }
                     r -= sp;
                 }
+                const uint32_t first = nv > 1 ? atile[i] : tile0 + ty0 * stride0 + tx0;
+                emit(j, am[i], first + row * astride[i] + col);
             }
-            // items without a table, one at a time: the warp evaluates 32
-            // rows at once, scans their spans and each of the item's lanes
-            // finds its row by binary search over the inclusive sums.  Every
-            // lane takes part in every shuffle (none sits behind a branch or
-            // a short-circuit).
-            const bool coop = valid && !tab;
-            uint32_t pending = __ballot_sync(kFull, coop);
-            while (pending) {
-                const int L = __ffs(pending) - 1;
-                const uint32_t mL = __shfl_sync(kFull, m, L);
-                const bool mine = coop && m == mL;
-                const FootprintEllipse EL = load_ellipse(ell, mL);
-                const uint2 rl = rect[mL];
-                const uint32_t ltx0 = rl.x & 0xffffu, lty0 = rl.x >> 16, ltx1 = rl.y & 0xffffu, lty1 = rl.y >> 16;
-                bool todo = mine;
-                uint32_t base = 0;
-                for (uint32_t row0 = lty0; row0 < lty1; row0 += 32) {
-                    const uint32_t row = row0 + lane;
-                    uint32_t cx = 0, sp = 0;
-                    if (row < lty1) {
-                        const uint2 cc = footprint_cols(EL, row, tile_w, tile_h, ltx0, ltx1);
-                        cx = cc.x;
-                        sp = cc.y - cc.x;
-                    }
-                    const uint32_t inc = warp_incl_scan(sp);
-                    const uint32_t total = __shfl_sync(kFull, inc, 31);
-                    const uint32_t rr = r - base;  // used only while todo (then r >= base)
+        }
+        // items without a table: one with more than kEmitThreads outputs in
+        // the chunk by all warps, 32 outputs each in turn, the others by one
+        // warp each
+        const uint32_t jend = min(j0 + kEmitChunk, K), nbig = s_nbig;
+        for (uint32_t b = 0; b < nbig; b++) {
+            const uint32_t m = s_big[b], off = vis_off[m], lo = max(off, j0), hi = min(off + vis_cnt[m], jend);
+            if (lo >= hi) continue;
+            const bool shared = hi - lo > (uint32_t)kEmitThreads;
+            if (!shared && (int)(b % (kEmitThreads / 32)) != warp) continue;
+            const uint32_t mine = lo + (shared ? 32u * warp : 0u) + lane, step = shared ? (uint32_t)kEmitThreads : 32u;
+            const FootprintEllipse E = load_ellipse(ell, m);
+            const uint2 rc = rect[m];
+            const uint32_t tx0 = rc.x & 0xffffu, ty0 = rc.x >> 16, tx1 = rc.y & 0xffffu, ty1 = rc.y >> 16;
+            const uint32_t stride = nv > 1 ? vis_stride[m] : stride0;
+            const uint32_t first = nv > 1 ? vis_tile[m] : tile0 + ty0 * stride0 + tx0;
+            uint32_t base = off;  // first output of the 32 rows
+            uint32_t j = mine;
+            for (uint32_t row0 = ty0; row0 < ty1 && base < hi; row0 += 32) {
+                const uint32_t row = row0 + lane;
+                uint32_t cx = 0, sp = 0;
+                if (row < ty1) {
+                    const uint2 cc = footprint_cols(E, row, tile_w, tile_h, tx0, tx1);
+                    cx = cc.x;
+                    sp = cc.y - cc.x;
+                }
+                const uint32_t inc = warp_incl_scan(sp);
+                const uint32_t end = base + __shfl_sync(kFull, inc, 31);
+                while (__any_sync(kFull, j < min(end, hi))) {
+                    const bool on = j < min(end, hi);
+                    const uint32_t rr = on ? j - base : 0u;
                     uint32_t k = 0;  // first lane whose inclusive sum exceeds rr
 #pragma unroll
-                    for (int step = 16; step; step >>= 1) {
-                        const uint32_t v = __shfl_sync(kFull, inc, k + step - 1);
-                        if (v <= rr) k += step;
+                    for (int s = 16; s; s >>= 1) {
+                        const uint32_t v = __shfl_sync(kFull, inc, k + s - 1);
+                        if (v <= rr) k += s;
                     }
-                    const uint32_t inc_k = __shfl_sync(kFull, inc, k), sp_k = __shfl_sync(kFull, sp, k);
-                    const uint32_t cx_k = __shfl_sync(kFull, cx, k);
-                    if (todo && rr < total) {
-                        ty = row0 + k;
-                        tx = cx_k + rr - (inc_k - sp_k);
-                        todo = false;
+                    const uint32_t inc_k = __shfl_sync(kFull, inc, k & 31), sp_k = __shfl_sync(kFull, sp, k & 31);
+                    const uint32_t cx_k = __shfl_sync(kFull, cx, k & 31);
+                    if (on) {
+                        emit(j, m, first + (row0 + k - ty0) * stride + (cx_k - tx0) + rr - (inc_k - sp_k));
+                        j += step;
                     }
-                    base += total;
-                    if (!__any_sync(kFull, todo)) break;
                 }
-                pending &= ~__ballot_sync(kFull, mine);
-            }
-            if (valid) {
-                const int view = nv == 1 ? 0 : view_of_item(views, nv, sgid[m]);
-                const uint32_t key = views[view].tile_base + ty * (uint32_t)views[view].tiles_x + tx;
-                keys[j] = key;
-                vals[j] = m;
-                const uint32_t d = key & (kRadix - 1u), sb = j / seg - sb0;
-                if (sb < (uint32_t)nsb) atomicAdd(&s_hist[sb][d], 1u);
-                else atomicAdd(&hist[(size_t)d * sort_G + sb0 + sb], 1u);
+                base = end;
             }
         }
         __syncthreads();
@@ -499,15 +529,31 @@ static_assert(kSortThreads == kRadix, "one thread per digit in the downsweep");
 
 template <int TILE>
 struct SortSmem {
-    uint32_t base[kRadix];                // running global offset per digit
     uint32_t warp_hist[kSortWarps][kRadix];
     uint32_t tile_start[kRadix];
+    uint32_t off[kRadix];                 // global position of a digit's run, less its tile_start
     uint32_t keys[TILE];
     uint32_t vals[TILE];
     uint32_t scan[33];
 };
 
-// NB: ballots per key in the ranking (the pass's digit width, or 8)
+// exclusive scan over the block's kSortThreads values, one barrier; smem: a
+// word per warp, not written again before the caller's next barrier
+__device__ __forceinline__ uint32_t sort_excl_scan(uint32_t v, uint32_t *smem) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t incl = warp_incl_scan(v);
+    if (lane == 31) smem[warp] = incl;
+    __syncthreads();
+    uint32_t before = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; w++) before += w < warp ? smem[w] : 0u;
+    return before + incl - v;
+}
+
+// NB: ballots per key in the ranking (the pass's digit width, or 8).  A
+// block's tiles follow one another, so a tile's global loads are started as
+// soon as the previous tile's keys have left the registers, and complete
+// behind its write-out; four barriers per tile.
 template <int ITEMS, int NB, bool kLateVals>
 __device__ __forceinline__ void radix_downsweep(const uint32_t *__restrict__ keys_in,
                                                 const uint32_t *__restrict__ vals_in, uint32_t *__restrict__ keys_out,
@@ -517,34 +563,37 @@ __device__ __forceinline__ void radix_downsweep(const uint32_t *__restrict__ key
     constexpr int kSortTile = kSortThreads * ITEMS;
     __shared__ SortSmem<kSortTile> S;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    {
-        // digit bases: exclusive prefix of the per-digit totals (one thread per digit)
-        uint32_t tot;
-        const uint32_t dbase = block_excl_scan(totals[tid], S.scan, &tot);
-        S.base[tid] = dbase + hist[tid * gridDim.x + blockIdx.x];
-    }
     uint32_t b0, b1;
     segment_of(min(*d_n, cap), gridDim.x, kSortTile, &b0, &b1);
+    // kLateVals: the values are read only when they are placed (below),
+    // so that a thread holds its keys and ranks but not its values
+    // meanwhile (64 registers: four CTAs per SM)
+    uint32_t key[ITEMS], val[kLateVals ? 1 : ITEMS];
+    const uint32_t mine = warp * (32 * ITEMS) + lane;  // the thread's first place in a tile
+    auto load = [&](uint32_t t0) {
+#pragma unroll
+        for (int j = 0; j < ITEMS; j++) {
+            const uint32_t pos = t0 + mine + j * 32;
+            key[j] = pos < b1 ? keys_in[pos] : 0u;
+            if constexpr (!kLateVals) val[j] = pos < b1 ? vals_in[pos] : 0u;
+        }
+    };
+    if (b0 < b1) load(b0);
+    // digit bases: exclusive prefix of the per-digit totals (one thread per
+    // digit); thread d keeps digit d's running global offset
+    uint32_t base = sort_excl_scan(totals[tid], S.scan) + hist[tid * gridDim.x + blockIdx.x];
+    __syncthreads();
     const uint32_t lt = lanemask_lt();
     for (uint32_t t0 = b0; t0 < b1; t0 += kSortTile) {
-        for (int k = tid; k < kSortWarps * kRadix; k += kSortThreads) (&S.warp_hist[0][0])[k] = 0;
-        __syncthreads();
-        // kLateVals: the values are read only when they are placed (below),
-        // so that a thread holds its keys and ranks but not its values
-        // meanwhile (64 registers: four CTAs per SM)
-        uint32_t key[ITEMS], val[kLateVals ? 1 : ITEMS], rank[ITEMS];
-        bool valid[ITEMS];
+        const uint32_t n = min(b1 - t0, (uint32_t)kSortTile);
+        for (int k = lane; k < kRadix; k += 32) S.warp_hist[warp][k] = 0;
+        __syncwarp();
+        uint32_t rank[ITEMS];
 #pragma unroll
         for (int j = 0; j < ITEMS; j++) {
-            const uint32_t pos = t0 + warp * (32 * ITEMS) + j * 32 + lane;
-            valid[j] = pos < b1;
-            key[j] = valid[j] ? keys_in[pos] : 0u;
-            if constexpr (!kLateVals) val[j] = valid[j] ? vals_in[pos] : 0u;
-        }
-#pragma unroll
-        for (int j = 0; j < ITEMS; j++) {
+            const bool valid = mine + j * 32 < n;
             const uint32_t d = (key[j] >> shift) & mask;
-            uint32_t peers = __ballot_sync(0xffffffffu, valid[j]);
+            uint32_t peers = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
             for (int bit = 0; bit < NB; bit++) {
                 const bool on = (d >> bit) & 1u;
@@ -552,49 +601,49 @@ __device__ __forceinline__ void radix_downsweep(const uint32_t *__restrict__ key
                 peers &= on ? b : ~b;
             }
             uint32_t before = 0;
-            if (valid[j]) before = S.warp_hist[warp][d];
+            if (valid) before = S.warp_hist[warp][d];
             __syncwarp();
-            if (valid[j] && (peers & lt) == 0) S.warp_hist[warp][d] = before + __popc(peers);
+            if (valid && (peers & lt) == 0) S.warp_hist[warp][d] = before + __popc(peers);
             __syncwarp();
             rank[j] = before + __popc(peers & lt);
         }
         __syncthreads();
         // per digit: exclusive offsets across warps, tile count, tile start
-        uint32_t tile_cnt = 0;
         {
             const int d = tid;  // kSortThreads == kRadix
+            uint32_t tile_cnt = 0;
 #pragma unroll
             for (int w = 0; w < kSortWarps; w++) {
                 const uint32_t c = S.warp_hist[w][d];
                 S.warp_hist[w][d] = tile_cnt;
                 tile_cnt += c;
             }
-            uint32_t tot;
-            S.tile_start[d] = block_excl_scan(tile_cnt, S.scan, &tot);
+            const uint32_t start = sort_excl_scan(tile_cnt, S.scan);
+            S.tile_start[d] = start;
+            S.off[d] = base - start;
+            base += tile_cnt;
         }
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < ITEMS; j++) {
-            if (!valid[j]) continue;
+            if (mine + j * 32 >= n) continue;
             const uint32_t d = (key[j] >> shift) & mask;
             const uint32_t p = S.tile_start[d] + S.warp_hist[warp][d] + rank[j];
             S.keys[p] = key[j];
-            if constexpr (kLateVals) S.vals[p] = vals_in[t0 + warp * (32 * ITEMS) + j * 32 + lane];
+            if constexpr (kLateVals) S.vals[p] = vals_in[t0 + mine + j * 32];
             else S.vals[p] = val[j];
         }
+        if (t0 + kSortTile < b1) load(t0 + kSortTile);
         __syncthreads();
-        const uint32_t nvalid = (b1 - t0) < (uint32_t)kSortTile ? (b1 - t0) : (uint32_t)kSortTile;
-        for (uint32_t p = tid; p < nvalid; p += kSortThreads) {
-            const uint32_t k = S.keys[p];
-            const uint32_t d = (k >> shift) & mask;
-            const uint32_t dst = S.base[d] + (p - S.tile_start[d]);
+        // (the next tile's writes to keys, vals, off lie behind its barriers)
+#pragma unroll 4
+        for (uint32_t p = tid; p < n; p += kSortThreads) {
+            const uint32_t k = S.keys[p], v = S.vals[p];
+            const uint32_t dst = S.off[(k >> shift) & mask] + p;
             keys_out[dst] = k;
-            vals_out[dst] = S.vals[p];
-            if (inv_out) inv_out[S.vals[p]] = dst;
+            vals_out[dst] = v;
+            if (inv_out) inv_out[v] = dst;
         }
-        __syncthreads();
-        S.base[tid] += tile_cnt;
-        __syncthreads();
     }
 }
 
@@ -606,7 +655,7 @@ __device__ __forceinline__ void radix_downsweep(const uint32_t *__restrict__ key
 // late reads' latency shows instead (a 3.3M-pair tile sort: 0.070 vs 0.061
 // ms).
 template <int ITEMS, int NB>
-__global__ void __launch_bounds__(kSortThreads) k_radix_downsweep(const uint32_t *__restrict__ keys_in,
+__global__ void __launch_bounds__(kSortThreads, ITEMS == kSortItems ? 3 : 4) k_radix_downsweep(const uint32_t *__restrict__ keys_in,
                                                                   const uint32_t *__restrict__ vals_in,
                                                                   uint32_t *__restrict__ keys_out,
                                                                   uint32_t *__restrict__ vals_out,
@@ -813,9 +862,9 @@ void scan_emit_pairs(const Params &p, void *temp, cudaStream_t s) {
     if (grid < 1) grid = 1;
     if (grid > (uint32_t)(8 * device_sm_count())) grid = 8 * device_sm_count();
     note_launch();
-    pdl_launch(k_expand_pairs, grid, kEmitThreads, 0, s, p.vis_off, p.vis_cnt, p.chunk_start, p.rect, p.rowtab, p.ell,
+    pdl_launch(k_expand_pairs<kEmitChunk>, grid, kEmitThreads, 0, s, p.vis_off, p.vis_cnt, p.chunk_start, p.rect, p.rowtab, p.ell,
                                                  p.tile_w, p.tile_h,
-                                                 p.sgid, p.views, p.n_views,
+                                                 p.vis_tile, p.vis_stride, p.views, p.n_views,
                                                  &p.counters[0], &p.counters[1], p.pair_capacity, p.pair_keys,
                                                  p.pair_vals, t.hist, sort_G, (uint32_t)(kSortThreads * sort_items));
 }
@@ -826,50 +875,92 @@ void scan_emit_pairs(const Params &p, void *temp, cudaStream_t s) {
 // to the atomics (each tile's result does not depend on when it runs).
 // walk (optional): order by the tiles' walk lengths instead (the adjoint:
 // each tile's largest last-blend position, which the forward recorded).
-// One block, any multiple of 64 threads.
-__device__ __forceinline__ void tile_order_block(const uint2 *__restrict__ ranges, const uint32_t *walk,
-                                                 uint32_t n_tiles, uint32_t *__restrict__ order) {
-    __shared__ uint32_t cnt[64];
+// One cluster of kOrderCtas CTAs (rank: this one's), which count their
+// shares of the tiles and read one another's counts; a warp adds once per
+// bucket it meets (with 55,000 tiles one CTA with an atomic per tile took 60
+// us, most tiles being in a few buckets).  Every CTA of the cluster calls.
+// CTAS = 1: one CTA without a cluster.
+constexpr int kOrderCtas = 8;
+
+template <int CTAS>
+__device__ __forceinline__ void tile_order(uint32_t rank, const uint2 *__restrict__ ranges,
+                                                   const uint32_t *walk, uint32_t n_tiles,
+                                                   uint32_t *__restrict__ order) {
+    __shared__ uint32_t cnt[64], place[64];
     __shared__ uint32_t smem[33];
     if (threadIdx.x < 64) cnt[threadIdx.x] = 0;
     __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const uint32_t stride = CTAS * blockDim.x, first = rank * blockDim.x + threadIdx.x;
+    // the lane's tile's bucket (64: none), and the lanes of its bucket
     auto bucket = [&](uint32_t t) {
+        if (t >= n_tiles) return 64;
         const uint32_t len = walk ? walk[t] : ranges[t].y - ranges[t].x;
-        const int b = min(63, (int)(log2f((float)len + 1.0f) * 3.0f));
-        return 63 - b;  // longest first
+        return 63 - min(63, (int)(lg2_approx((float)len + 1.0f) * 3.0f));  // longest first
     };
-    for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x) atomicAdd(&cnt[bucket(t)], 1u);
-    __syncthreads();
+    auto take = [&](uint32_t *counts, int b, uint32_t peers) {
+        uint32_t base = 0;
+        if (b < 64 && lane == __ffs(peers) - 1) base = atomicAdd(&counts[b], __popc(peers));
+        return __shfl_sync(0xffffffffu, base, __ffs(peers) - 1) + __popc(peers & lanemask_lt());
+    };
+    const uint32_t rounds = (n_tiles + stride - 1) / stride;
+    for (uint32_t k = 0; k < rounds; k++) {
+        const int b = bucket(first + k * stride);
+        take(cnt, b, __match_any_sync(0xffffffffu, b));
+    }
+    if constexpr (CTAS > 1) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
+    // places: the longer buckets of all CTAs, then this bucket's of the CTAs before
+    uint32_t all = 0, before = 0;
+    if (threadIdx.x < 64) {
+        if constexpr (CTAS > 1) {
+            for (uint32_t c = 0; c < CTAS; c++) {
+                const uint32_t v = cooperative_groups::this_cluster().map_shared_rank(cnt, c)[threadIdx.x];
+                all += v;
+                before += c < rank ? v : 0u;
+            }
+        } else {
+            all = cnt[threadIdx.x];
+        }
+    }
     uint32_t tot;
-    const uint32_t v = threadIdx.x < 64 ? cnt[threadIdx.x] : 0u;
-    const uint32_t ex = block_excl_scan(v, smem, &tot);
-    if (threadIdx.x < 64) cnt[threadIdx.x] = ex;
-    __syncthreads();
-    for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x) order[atomicAdd(&cnt[bucket(t)], 1u)] = t;
+    const uint32_t ex = block_excl_scan(all, smem, &tot);
+    if (threadIdx.x < 64) place[threadIdx.x] = ex + before;
+    // no CTA leaves, or counts again, while another reads its counts
+    if constexpr (CTAS > 1) cooperative_groups::this_cluster().sync();
+    else __syncthreads();
+    for (uint32_t k = 0; k < rounds; k++) {
+        const uint32_t t = first + k * stride;
+        const int b = bucket(t);
+        const uint32_t at = take(place, b, __match_any_sync(0xffffffffu, b));
+        if (b < 64) order[at] = t;
+    }
 }
 
-__global__ void __launch_bounds__(1024) k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles,
-                                                     uint32_t *__restrict__ order, uint32_t *__restrict__ walk) {
+__global__ void __cluster_dims__(kOrderCtas, 1, 1) __launch_bounds__(1024)
+    k_tile_order(const uint2 *__restrict__ ranges, uint32_t n_tiles, uint32_t *__restrict__ order,
+                 uint32_t *__restrict__ walk) {
     pdl_enter();
     if (walk)
-        for (uint32_t t = threadIdx.x; t < n_tiles; t += blockDim.x) walk[t] = 0u;
-    tile_order_block(ranges, nullptr, n_tiles, order);
+        for (uint32_t t = blockIdx.x * 1024u + threadIdx.x; t < n_tiles; t += kOrderCtas * 1024u) walk[t] = 0u;
+    tile_order<kOrderCtas>(blockIdx.x, ranges, nullptr, n_tiles, order);
 }
 
 // The adjoint's first kernel: rows [0, *d_m) of the image-space gradients
-// zeroed (the visible items', which the adjoint accumulates) by all blocks
+// zeroed (the visible items', which the adjoint accumulates) by all clusters
 // but the last, which orders the tiles by their walk lengths and resets the
 // per-item adjoint's chunk ticket (counters[3]).
-__global__ void __launch_bounds__(1024) k_bwd_prep(double *__restrict__ g2m, float *__restrict__ g2d,
+__global__ void __cluster_dims__(kOrderCtas, 1, 1) __launch_bounds__(1024) k_bwd_prep(double *__restrict__ g2m, float *__restrict__ g2d,
                                                   const uint32_t *d_m, const uint32_t *walk, uint32_t n_tiles,
                                                   uint32_t *__restrict__ order, uint32_t *ticket) {
     pdl_enter();
-    if (blockIdx.x == gridDim.x - 1) {
-        if (threadIdx.x == 0) *ticket = 0u;  // the per-item adjoint's chunk ticket
-        tile_order_block(nullptr, walk, n_tiles, order);
+    if (blockIdx.x + kOrderCtas >= gridDim.x) {
+        const uint32_t rank = blockIdx.x + kOrderCtas - gridDim.x;
+        if (rank == 0 && threadIdx.x == 0) *ticket = 0u;  // the per-item adjoint's chunk ticket
+        tile_order<kOrderCtas>(rank, nullptr, walk, n_tiles, order);
         return;
     }
-    const size_t M = *d_m, stride = (size_t)(gridDim.x - 1) * blockDim.x;
+    const size_t M = *d_m, stride = (size_t)(gridDim.x - kOrderCtas) * blockDim.x;
     const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     for (size_t k = first; k < 3 * M; k += stride) g2m[k] = 0.0;
     float4 *rows = reinterpret_cast<float4 *>(g2d);
@@ -879,12 +970,13 @@ __global__ void __launch_bounds__(1024) k_bwd_prep(double *__restrict__ g2m, flo
 void launch_tile_order(const Params &p, cudaStream_t s) {
     if (p.total_tiles == 0) return;
     note_launch();
-    pdl_launch(k_tile_order, 1, 1024, 0, s, p.ranges, p.total_tiles, p.tile_order, p.tile_walk);
+    pdl_launch(k_tile_order, kOrderCtas, 1024, 0, s, p.ranges, p.total_tiles, p.tile_order, p.tile_walk);
 }
 
 void launch_bwd_prep(const Params &p, const uint32_t *walk, uint32_t *order, cudaStream_t s) {
     note_launch();
-    pdl_launch(k_bwd_prep, device_sm_count() + 1, 1024, 0, s, p.g2m, p.g2d, (const uint32_t *)&p.counters[0], walk,
+    const int zero_ctas = (device_sm_count() + kOrderCtas - 1) / kOrderCtas * kOrderCtas;  // whole clusters
+    pdl_launch(k_bwd_prep, zero_ctas + kOrderCtas, 1024, 0, s, p.g2m, p.g2d, (const uint32_t *)&p.counters[0], walk,
                p.total_tiles, order, &p.counters[3]);
 }
 
