@@ -76,24 +76,6 @@ __global__ void __launch_bounds__(256, 4) k_finalize(Params P) {
             P.vis_tile[m] = V.tile_base + F.ty0 * (uint32_t)V.tiles_x + F.tx0;
             P.vis_stride[m] = (uint32_t)V.tiles_x;
         }
-        float dx = F.mut.x - V.campos[0], dy = F.mut.y - V.campos[1], dz = F.mut.z - V.campos[2];
-        const float inv = 1.0f / sqrtf(dx * dx + dy * dy + dz * dz);
-        dx *= inv; dy *= inv; dz *= inv;
-        float Y[16], dY[16][3];
-        sh_eval<D, false>(dx, dy, dz, Y, dY);
-        float sh[3 * K];
-        load_floats<3 * K>(V.sh + (size_t)i * K * 3, sh, aligned16(V.sh));
-        float rgb[3] = {0.5f, 0.5f, 0.5f};
-#pragma unroll
-        for (int k = 0; k < K; k++) {
-            rgb[0] += sh[3 * k] * Y[k];
-            rgb[1] += sh[3 * k + 1] * Y[k];
-            rgb[2] += sh[3 * k + 2] * Y[k];
-        }
-        const float z = __uint_as_float(P.szkey[m]);
-        P.rec[3 * (size_t)m + 0] = make_float4(F.u, F.v, F.ca, F.cb);
-        P.rec[3 * (size_t)m + 1] = make_float4(F.cc, F.ot, z, F.hx);
-        P.rec[3 * (size_t)m + 2] = make_float4(fmaxf(rgb[0], 0.0f), fmaxf(rgb[1], 0.0f), fmaxf(rgb[2], 0.0f), F.hy);
         P.rect[m] = make_uint2(F.tx0 | (F.ty0 << 16), F.tx1 | (F.ty1 << 16));
         // tiles of the rectangle that the footprint ellipse meets
         const FootprintEllipse E = footprint_ellipse(F.u, F.v, F.ca, F.cb, F.cc, F.ot);
@@ -112,6 +94,24 @@ __global__ void __launch_bounds__(256, 4) k_finalize(Params P) {
         }
         if (tab) P.rowtab[m] = make_uint4(w0, w1, w2, w3);
         P.vis_cnt[m] = cnt;
+        float dx = F.mut.x - V.campos[0], dy = F.mut.y - V.campos[1], dz = F.mut.z - V.campos[2];
+        const float inv = 1.0f / sqrtf(dx * dx + dy * dy + dz * dz);
+        dx *= inv; dy *= inv; dz *= inv;
+        float Y[16], dY[16][3];
+        sh_eval<D, false>(dx, dy, dz, Y, dY);
+        float sh[3 * K];
+        load_floats<3 * K>(V.sh + (size_t)i * K * 3, sh, aligned16(V.sh));
+        float rgb[3] = {0.5f, 0.5f, 0.5f};
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            rgb[0] += sh[3 * k] * Y[k];
+            rgb[1] += sh[3 * k + 1] * Y[k];
+            rgb[2] += sh[3 * k + 2] * Y[k];
+        }
+        const float z = __uint_as_float(P.szkey[m]);
+        P.rec[3 * (size_t)m + 0] = make_float4(F.u, F.v, F.ca, F.cb);
+        P.rec[3 * (size_t)m + 1] = make_float4(F.cc, F.ot, z, F.hx);
+        P.rec[3 * (size_t)m + 2] = make_float4(fmaxf(rgb[0], 0.0f), fmaxf(rgb[1], 0.0f), fmaxf(rgb[2], 0.0f), F.hy);
     }
 }
 

@@ -8,14 +8,16 @@
 namespace pvg {
 namespace {
 
-// Resident warps per SM that the registers are held to (no spills: 16 warps
-// of 126 registers with eight pixels per lane), and entries whose alphas are
-// evaluated together, by pixels per lane: with two pixels a lane the walk is
-// latency-bound and overlaps four, with eight the pixels are parallel enough.
+// Resident warps per SM that the registers are held to (16 warps of 126
+// registers with eight pixels per lane), and entries whose alphas are
+// evaluated together, by pixels per lane: with two or four pixels a lane the
+// longest walk bounds the frame and four evaluations overlap its latencies
+// (1242x375, four pixels: 162 us one by one, 147 us by twos, 139 us by
+// fours), with eight the pixels are parallel enough.
 template <int PX>
 struct BwdTune {
     static constexpr int kWarps = PX == 2 ? 20 : 16;
-    static constexpr int kUnroll = PX == 8 ? 1 : PX == 4 ? 2 : 4;
+    static constexpr int kUnroll = PX == 8 ? 1 : 4;
 };
 // Blocks of 256 (128) pixels per SM from which a lane takes eight (four)
 // pixels.  Eight make an entry's fixed work (its staged loads, the warp sum,
@@ -54,8 +56,12 @@ struct TermBuffer {
 template <int NT>
 __device__ __forceinline__ void flush_terms(const TermBuffer<NT> &buf, const Staged &S, int base, uint32_t valid,
                                             int lane, const Params &P) {
-    __syncwarp();
     const int slot = lane >> 3, half = (lane >> 2) & 1, sub = lane & 3;
+    // the slot's entry: loaded ahead of the sums
+    const size_t m = S.m[base + slot];
+    const float4 ab = S.a[base + slot], gb = S.d[base + slot];  // (u, a', b', -), (g, g, b, b)
+    const float cc = S.b[base + slot].z, red = S.c[base + slot].z;
+    __syncwarp();
     const float4 *h = &buf.h[slot][half][sub];
     float2 a, b;
 #pragma unroll
@@ -64,48 +70,40 @@ __device__ __forceinline__ void flush_terms(const TermBuffer<NT> &buf, const Sta
         a = j ? add2(a, make_float2(v.x, v.y)) : make_float2(v.x, v.y);
         b = j ? add2(b, make_float2(v.z, v.w)) : make_float2(v.z, v.w);
     }
-    const bool hi2 = sub & 2, hi1 = sub & 1;
-    const float c0 = (hi2 ? b.x : a.x) + __shfl_xor_sync(0xffffffffu, hi2 ? a.x : b.x, 2);
-    const float c1 = (hi2 ? b.y : a.y) + __shfl_xor_sync(0xffffffffu, hi2 ? a.y : b.y, 2);
-    float d = (hi1 ? c1 : c0) + __shfl_xor_sync(0xffffffffu, hi1 ? c0 : c1, 1);
     float s[NT - 8];
 #pragma unroll
     for (int t = 0; t < NT - 8; t++) {
         const float4 v = reinterpret_cast<const float4 *>(&buf.e[t][0][0])[lane];
         s[t] = (v.x + v.y) + (v.z + v.w);
+    }
+    const bool hi2 = sub & 2, hi1 = sub & 1;
+    const float c0 = (hi2 ? b.x : a.x) + __shfl_xor_sync(0xffffffffu, hi2 ? a.x : b.x, 2);
+    const float c1 = (hi2 ? b.y : a.y) + __shfl_xor_sync(0xffffffffu, hi2 ? a.y : b.y, 2);
 #pragma unroll
-        for (int o = 1; o < 8; o <<= 1) s[t] += __shfl_xor_sync(0xffffffffu, s[t], o);
-    }
-    // half 0 holds m_xx, m_xy, m_yy, m_0, half 1 m_x, m_y, r, g
+    for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+        for (int t = 0; t < NT - 8; t++) s[t] += __shfl_xor_sync(0xffffffffu, s[t], o);
+    const float d = (hi1 ? c1 : c0) + __shfl_xor_sync(0xffffffffu, hi1 ? c0 : c1, 1);
     const float q = __shfl_xor_sync(0xffffffffu, d, 1);
-    if ((valid >> slot) & 1u) {
-        const size_t m = S.m[base + slot];
-        const float4 gb = S.d[base + slot], ab = S.a[base + slot];
-        if (half == 0 && sub < 3) {
-            // the second moments in 64 bits: the per-item adjoint's products
-            // with the conic cancel and amplify the rounding of their sums
-            if (d != 0.f) atomicAdd(P.g2m + 3 * m + sub, (double)d);
-        } else {
-            bool keep = d != 0.f;
-            int t = kG2dColour + sub - 2;
-            if (half == 0) {
-                t = kG2dPower;
-            } else if (sub < 2) {
-                // gradients of u and v (conic a = -2 ln 2 a', b = -ln 2 b'),
-                // here and not from the moments' totals: a m_x + b m_y cancels
-                const float own = sub == 0 ? ab.y : S.b[base + slot].z;
-                d = -0.6931471805599453f * (2.0f * own * d + ab.z * q);
-                keep = d != 0.f;
-                t = sub;
-            } else {  // the colours: none where the forward clamped
-                keep = keep && (sub == 2 ? S.c[base + slot].z : gb.x) > 0.f;
-            }
-            if (keep) atomicAdd(P.g2d + kG2dRow * m + t, d);
-        }
-        if ((lane & 7) == 0 && s[0] != 0.f && gb.z > 0.f) atomicAdd(P.g2d + kG2dRow * m + kG2dColour + 2, s[0]);
-        if (NT == 10 && (lane & 7) == 1 && s[NT - 9] != 0.f) atomicAdd(P.g2d + kG2dRow * m + kG2dDepth, s[NT - 9]);
-    }
-    __syncwarp();
+    __syncwarp();  // the buffer is free
+    // Half 0 holds m_xx, m_xy, m_yy, m_0, half 1 m_x, m_y, r, g; every lane
+    // but one adds one float (a lane of the second moments the colour b or
+    // the depth), three lanes a moment in 64 bits: the per-item adjoint's
+    // products with the conic cancel and amplify the rounding of their sums.
+    // The gradients of u and v (conic a = -2 ln 2 a', b = -ln 2 b') are taken
+    // here and not from the moments' totals, since a m_x + b m_y cancels too.
+    // No colour term where the forward clamped.  (Two atomics for the whole
+    // warp: one per kind of term in branches of their own took 7 us more
+    // on the 1242x375 frame and 33 us on a sparse 961x641 one.)
+    const float uv = -0.6931471805599453f * (2.0f * (sub == 0 ? ab.y : cc) * d + ab.z * q);
+    const float gate = half == 0 ? (sub == 0 ? gb.z : 1.0f) : sub == 2 ? red : sub == 3 ? gb.x : 1.0f;
+    const float v = half == 0 ? (sub == 0 ? s[0] : sub == 3 ? d : NT == 10 && sub == 1 ? s[NT - 9] : 0.0f)
+                              : (sub < 2 ? uv : d);
+    const int t = half == 0 ? (sub == 0 ? kG2dColour + 2 : sub == 1 ? kG2dDepth : kG2dPower)
+                            : (sub < 2 ? sub : kG2dColour + sub - 2);
+    const bool on = (valid >> slot) & 1u;
+    if (on && v != 0.f && gate > 0.f) atomicAdd(P.g2d + kG2dRow * m + t, v);
+    if (on && half == 0 && sub < 3 && d != 0.f) atomicAdd(P.g2m + 3 * m + sub, (double)d);
 }
 
 // The channels' gradients of up to U entries, summed over the warp and added
@@ -164,7 +162,47 @@ struct PixelAdjoint {
     uint32_t last;
 };
 
-__device__ __forceinline__ PixelAdjoint pixel_adjoint(const Params &P, const ViewDesc &V, int px, int py) {
+// dL/d(sky texels) of a lane's pixels, one after another: vertically adjacent
+// pixels mostly sample the same four texels, whose shares are added up here
+// and reach memory once (a 961 pixels wide 50 degree view of a 256-texel face
+// has seven pixels to a texel)
+struct SkyScatter {
+    size_t first = ~(size_t)0, last = 0;  // indices of the corners (0, 0) and (1, 1), which fix the other two
+    size_t idx[4];
+    float acc[4][3];
+
+    __device__ __forceinline__ void add(const ViewDesc &V, const size_t (&ti)[4], const float (&tw)[4], float wo,
+                                        const float (&gc)[3]) {
+        if (ti[0] != first || ti[3] != last) {
+            flush(V);
+            first = ti[0];
+            last = ti[3];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                idx[q] = ti[q];
+#pragma unroll
+                for (int c = 0; c < 3; c++) acc[q][c] = 0.f;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+#pragma unroll
+            for (int c = 0; c < 3; c++)
+                if (tw[q] != 0.f && gc[c] != 0.f) acc[q][c] += tw[q] * wo * gc[c];
+    }
+    __device__ __forceinline__ void flush(const ViewDesc &V) {
+        if (first == ~(size_t)0) return;
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+#pragma unroll
+            for (int c = 0; c < 3; c++)
+                if (acc[q][c] != 0.f) atomicAdd(V.g_sky + idx[q] + c, acc[q][c]);
+        first = ~(size_t)0;
+    }
+};
+
+__device__ __forceinline__ PixelAdjoint pixel_adjoint(const Params &P, const ViewDesc &V, int px, int py,
+                                                      SkyScatter &sky) {
     PixelAdjoint a;
     a.T = 1.0f;
     a.gC0 = a.gC1 = a.gC2 = a.gD = a.gO = 0.f;
@@ -196,11 +234,8 @@ __device__ __forceinline__ PixelAdjoint pixel_adjoint(const Params &P, const Vie
             const float f = tw[0] * V.sky[ti[0] + c] + tw[1] * V.sky[ti[1] + c] + tw[2] * V.sky[ti[2] + c] +
                             tw[3] * V.sky[ti[3] + c];
             a.gO -= gc[c] * f;
-            if (V.g_sky && gc[c] != 0.f)
-#pragma unroll
-                for (int q = 0; q < 4; q++)
-                    if (tw[q] != 0.f) atomicAdd(V.g_sky + ti[q] + c, tw[q] * wo * gc[c]);
         }
+        if (V.g_sky) sky.add(V, ti, tw, wo, gc);
         a.S = 0.f;
     }
     return a;
@@ -229,11 +264,13 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
     float2 S[NP];  // suffix sum of X_j alpha_j T_j
     uint32_t last[PX];
     uint32_t walk = 0;
+    SkyScatter sky;
     bool odd = false;  // non-finite or huge output gradients: pixels one at a time
 #pragma unroll
     for (int q = 0; q < NP; q++) {
         fy[q] = make_float2((float)(G.py0 + 2 * q) + 0.5f, (float)(G.py0 + 2 * q + 1) + 0.5f);
-        const PixelAdjoint a = pixel_adjoint(P, V, G.px, G.py0 + 2 * q), b = pixel_adjoint(P, V, G.px, G.py0 + 2 * q + 1);
+        const PixelAdjoint a = pixel_adjoint(P, V, G.px, G.py0 + 2 * q, sky);
+        const PixelAdjoint b = pixel_adjoint(P, V, G.px, G.py0 + 2 * q + 1, sky);
         T[q] = make_float2(a.T, b.T);
         S[q] = make_float2(a.S, b.S);
         nC0[q] = make_float2(-a.gC0, -b.gC0);
@@ -247,6 +284,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
         for (const PixelAdjoint &e : {a, b})
             odd |= !(fabsf(e.gC0) + fabsf(e.gC1) + fabsf(e.gC2) + fabsf(e.gD) + fabsf(e.gO) + fabsf(e.S) < 1e15f);
     }
+    sky.flush(V);
     float2 nF[NP][NG > 0 ? 4 * NG : 1];  // output gradients of the extra channels (negated)
     if constexpr (NG > 0) {
         const size_t HW = (size_t)V.W * V.H;
