@@ -14,6 +14,7 @@
 //   c  k_composite          images + per-pixel T and last position
 // Backward: k_composite_bwd (image-space gradients per record) and
 // k_preprocess_bwd (parameter gradients).
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -308,7 +309,8 @@ extern "C" pvg_status_t pvg_create(pvg_ctx_t **ctx, const pvg_config_t *cfg) {
     PVG_TRY(check_config(&c));
     pvg_ctx *x = new pvg_ctx();
     x->cfg = c;
-    if (cudaGetDevice(&x->device) != cudaSuccess || set_sh_constants() != cudaSuccess) {
+    if (cudaGetDevice(&x->device) != cudaSuccess || set_sh_constants() != cudaSuccess ||
+        set_small_frame_smem() != cudaSuccess) {
         g_last_error = cudaGetErrorString(cudaGetLastError());
         delete x;
         return PVG_ERR_CUDA;
@@ -572,6 +574,12 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
     PVG_TRY(ensure_c(f->pix_T, sizeof(float) * pix, capturing));
     PVG_TRY(ensure_c(f->pix_last, sizeof(uint32_t) * pix, capturing));
     PVG_TRY(ensure_c(f->pix_neval, sizeof(uint32_t) * 2 * (size_t)pix, capturing));
+    const bool small = NV <= kSmallFrameItems && tiles <= kSmallFrameTiles;  // one CTA per sorting stage
+    if (small)
+        PVG_TRY(ensure_c(x->chunk_start,
+                         sizeof(uint32_t) * small_emit_chunks(NV, tiles, x->cfg.sync_sizes ? 0xffffffffu
+                                                                                           : (uint32_t)x->cfg.pair_capacity),
+                         capturing));
     uint32_t pair_cap;
     if (x->cfg.sync_sizes) {
         pair_cap = (uint32_t)(f->pair_vals.bytes / sizeof(uint32_t));
@@ -656,10 +664,14 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
         // invisible items from the compaction, the visible ones' from the
         // sort's last pass; the compaction also counts the sort's first
         // digit histogram
-        compact_visible(p, p.szkey, p.sgid, p.inv, x->temp.p, s);
         bool in_alt = false;
-        radix_sort_pairs(p.szkey, p.sgid, ptr<uint32_t>(x->alt_keys), ptr<uint32_t>(x->alt_vals), &p.counters[0], NV,
-                         0, 31, x->temp.p, s, &in_alt, p.inv, true);
+        if (small) {
+            small_depth_sort(p, s);
+        } else {
+            compact_visible(p, p.szkey, p.sgid, p.inv, x->temp.p, s);
+            radix_sort_pairs(p.szkey, p.sgid, ptr<uint32_t>(x->alt_keys), ptr<uint32_t>(x->alt_vals), &p.counters[0],
+                             NV, 0, 31, x->temp.p, s, &in_alt, p.inv, true);
+        }
         if (in_alt) {  // 31 bits = 4 passes: never taken, kept for safety
             PVG_CUDA(cudaMemcpyAsync(p.szkey, x->alt_keys.p, sizeof(uint32_t) * NV, cudaMemcpyDeviceToDevice, s));
             PVG_CUDA(cudaMemcpyAsync(p.sgid, x->alt_vals.p, sizeof(uint32_t) * NV, cudaMemcpyDeviceToDevice, s));
@@ -671,7 +683,9 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
         tm.end(PVG_STAGE_FINALIZE, s);
         tm.begin(PVG_STAGE_PAIRS, s);
         p.pair_capacity = x->cfg.sync_sizes ? 0xffffffffu : pair_cap;
-        scan_count_pairs(p, x->temp.p, s);
+        p.chunk_start = ptr<uint32_t>(x->chunk_start);
+        if (small) small_count_pairs(p, s);
+        else scan_count_pairs(p, x->temp.p, s);
         if (x->cfg.sync_sizes) {
             PVG_CUDA(cudaMemcpyAsync(x->h_pinned, &p.counters[1], sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
             PVG_CUDA(cudaStreamSynchronize(s));
@@ -680,7 +694,7 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
             PVG_TRY(ensure_c(x->pair_keys, sizeof(uint32_t) * (size_t)K, capturing));
             PVG_TRY(ensure_c(x->pair_keys2, sizeof(uint32_t) * (size_t)K, capturing));
             PVG_TRY(ensure_c(x->pair_vals2, sizeof(uint32_t) * (size_t)K, capturing));
-            PVG_TRY(ensure_c(x->chunk_start, sizeof(uint32_t) * emit_chunks(K), capturing));
+            if (!small) PVG_TRY(ensure_c(x->chunk_start, sizeof(uint32_t) * emit_chunks(K), capturing));
             pair_cap = K;
         }
         p.pair_capacity = pair_cap;
@@ -697,19 +711,27 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
             E_vals = ptr<uint32_t>(x->pair_vals2);
             F_vals = ptr<uint32_t>(f->pair_vals);
         }
+        // small: one CTA sorts up to kSmallFrameItems pairs, from either buffer into f->pair_vals
+        const bool small_tiles = small && pair_cap <= kSmallFrameItems;
+        if (small_tiles) E_vals = ptr<uint32_t>(x->pair_vals2);
         p.pair_keys = E_keys;
         p.pair_vals = E_vals;
-        scan_emit_pairs(p, x->temp.p, s);
+        if (small) small_emit_pairs(p, x->temp.p, !small_tiles, s);
+        else scan_emit_pairs(p, x->temp.p, s);
         tm.end(PVG_STAGE_PAIRS, s);
         tm.begin(PVG_STAGE_TILE_SORT, s);
-        bool t_alt = false;
-        // the first digit pass's histogram was counted by the expansion
-        radix_sort_pairs(E_keys, E_vals, F_keys, F_vals, &p.counters[1], pair_cap, 0, tbits, x->temp.p, s, &t_alt,
-                         nullptr, true);
-        p.pair_keys = t_alt ? F_keys : E_keys;
-        p.pair_vals = ptr<uint32_t>(f->pair_vals);
-        launch_ranges(p, s);
-        launch_tile_order(p, s);
+        if (small_tiles) {
+            small_tile_sort(p, ptr<uint32_t>(f->pair_vals), tbits, s);
+        } else {
+            bool t_alt = false;
+            // the first digit pass's histogram was counted by the expansion
+            radix_sort_pairs(E_keys, E_vals, F_keys, F_vals, &p.counters[1], pair_cap, 0, tbits, x->temp.p, s, &t_alt,
+                             nullptr, true);
+            p.pair_keys = t_alt ? F_keys : E_keys;
+            p.pair_vals = ptr<uint32_t>(f->pair_vals);
+            launch_ranges(p, s);
+            launch_tile_order(p, s);
+        }
         tm.end(PVG_STAGE_TILE_SORT, s);
     } else {
         PVG_CUDA(cudaMemsetAsync(p.ranges, 0, sizeof(uint2) * tiles, s));
@@ -801,7 +823,9 @@ pvg_status_t serve_reserve(pvg_ctx_t *x, pvg_frame_t *f, uint64_t items, uint64_
     PVG_TRY(ensure(f->pix_neval, sizeof(uint32_t) * 2 * pix));
     for (DevBuf *b : {&f->pair_vals, &x->pair_keys, &x->pair_keys2, &x->pair_vals2})
         PVG_TRY(ensure(*b, sizeof(uint32_t) * pairs));
-    PVG_TRY(ensure(x->chunk_start, sizeof(uint32_t) * emit_chunks((uint32_t)pairs)));
+    PVG_TRY(ensure(x->chunk_start, sizeof(uint32_t) * std::max(emit_chunks((uint32_t)pairs),
+                                                               small_emit_chunks(kSmallFrameItems, kSmallFrameTiles,
+                                                                                 (uint32_t)pairs))));
     PVG_TRY(ensure(f->stage_fwd->dev, sizeof(ViewDesc) * (size_t)max_views));
     return PVG_OK;
 }

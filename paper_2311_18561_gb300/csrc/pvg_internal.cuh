@@ -489,6 +489,17 @@ void radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32
 void scan_count_pairs(const Params &p, void *temp, cudaStream_t s);
 void scan_emit_pairs(const Params &p, void *temp, cudaStream_t s);
 size_t emit_chunks(uint32_t capacity);
+// Small frames: the same stages, one CTA each.  At most kSmallFrameItems
+// items; the tile sort also at most as many pairs of capacity.
+constexpr uint32_t kSmallFrameItems = 8192, kSmallFrameTiles = 65536;
+constexpr uint32_t kSmallOrderTiles = 8192;  // above it the launch order is the cluster's
+cudaError_t set_small_frame_smem();
+size_t small_emit_chunks(uint64_t n_items, uint64_t tiles, uint32_t capacity);
+void small_depth_sort(const Params &p, cudaStream_t s);
+void small_count_pairs(const Params &p, cudaStream_t s);
+// count_digits: the general tile sort follows (its first digit histogram)
+void small_emit_pairs(const Params &p, void *temp, bool count_digits, cudaStream_t s);
+void small_tile_sort(const Params &p, uint32_t *vals_out, int bits, cudaStream_t s);
 void launch_ranges(const Params &p, cudaStream_t s);
 // the compositor's launch order; also zeroes p.tile_walk (if given), into
 // which the compositor's warps take maxima

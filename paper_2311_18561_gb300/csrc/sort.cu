@@ -48,9 +48,10 @@ constexpr uint32_t kSmallSort = 4u << 20;
 constexpr uint32_t kLateSortKeys = 12u << 20;  // capacity from which the wide sort reads values late
 constexpr int kRadix = kSortRadix;
 
-constexpr uint32_t kEmitChunk = 2048;  // pair outputs per expansion chunk
+constexpr uint32_t kEmitChunk = 2048;      // pair outputs per expansion chunk
+constexpr uint32_t kEmitChunkSmall = 512;  // of the small frames
 constexpr int kEmitThreads = 256;
-static_assert(kEmitChunk % kEmitThreads == 0, "whole warps per expansion pass");
+static_assert(kEmitChunk % kEmitThreads == 0 && kEmitChunkSmall % kEmitThreads == 0, "whole warps per expansion pass");
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
@@ -965,6 +966,254 @@ __global__ void __cluster_dims__(kOrderCtas, 1, 1) __launch_bounds__(1024) k_bwd
     for (size_t k = first; k < 3 * M; k += stride) g2m[k] = 0.0;
     float4 *rows = reinterpret_cast<float4 *>(g2d);
     for (size_t k = first; k < kG2dRow / 4 * M; k += stride) rows[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// ---------------------------------------------------------------- small frames
+//
+// With at most kSmallFrameItems items (and pairs) the general passes are a
+// chain of some twenty launches of a few microseconds each that leave the
+// chip idle; one CTA does each stage's work in shared memory instead: the
+// compaction and depth sort (14 launches), the pair count scan (3), the tile
+// sort with ranges and launch order (4 to 7).  Same order: stable passes over
+// items in gid order, pairs in depth order.
+namespace {
+
+constexpr int kOneThreads = 1024, kOneWarps = kOneThreads / 32;
+constexpr int kOneItems = (int)kSmallFrameItems / kOneThreads;  // keys per thread at most
+static_assert(kOneItems * kOneThreads == (int)kSmallFrameItems && kSmallFrameItems <= 65536, "16-bit values");
+
+struct OneSmem {
+    uint32_t keys[kSmallFrameItems];
+    uint16_t vals[kSmallFrameItems];
+    uint16_t hist[kOneWarps][kRadix];
+    uint32_t start[kRadix];
+    uint32_t scan[33];
+};
+
+// Stable LSD sort of S.keys / S.vals [0, n) by key bits [0, bits); the whole
+// CTA calls, the arrays written and synchronised before.
+__device__ __forceinline__ void one_cta_sort(OneSmem &S, uint32_t n, int bits) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t per = (n + kOneThreads - 1) / kOneThreads;  // keys per thread
+    const uint32_t mine = warp * per * 32 + lane;
+    const uint32_t lt = lanemask_lt();
+    for (int shift = 0; shift < bits; shift += 8) {
+        const uint32_t mask = bits - shift >= 8 ? 255u : (1u << (bits - shift)) - 1u;
+        for (int k = lane; k < kRadix; k += 32) S.hist[warp][k] = 0;
+        __syncwarp();
+        uint32_t key[kOneItems], rank[kOneItems];
+        uint16_t val[kOneItems];
+#pragma unroll
+        for (int j = 0; j < kOneItems; j++) {
+            if ((uint32_t)j >= per) break;
+            const uint32_t pos = mine + j * 32;
+            const bool valid = pos < n;
+            key[j] = valid ? S.keys[pos] : 0u;
+            val[j] = valid ? S.vals[pos] : (uint16_t)0;
+            const uint32_t d = (key[j] >> shift) & mask;
+            uint32_t peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+            for (int bit = 0; bit < 8; bit++) {
+                const bool on = (d >> bit) & 1u;
+                const uint32_t b = __ballot_sync(0xffffffffu, on);
+                peers &= on ? b : ~b;
+            }
+            uint32_t before = 0;
+            if (valid) before = S.hist[warp][d];
+            __syncwarp();
+            if (valid && (peers & lt) == 0) S.hist[warp][d] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+            rank[j] = before + __popc(peers & lt);
+        }
+        __syncthreads();
+        uint32_t cnt = 0;
+        if (tid < kRadix) {
+            uint32_t c[kOneWarps];
+#pragma unroll
+            for (int w = 0; w < kOneWarps; w++) c[w] = S.hist[w][tid];
+#pragma unroll
+            for (int w = 0; w < kOneWarps; w++) {
+                S.hist[w][tid] = (uint16_t)cnt;
+                cnt += c[w];
+            }
+        }
+        uint32_t tot;
+        const uint32_t ex = block_excl_scan(cnt, S.scan, &tot);
+        if (tid < kRadix) S.start[tid] = ex;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kOneItems; j++) {
+            if ((uint32_t)j >= per) break;
+            if (mine + j * 32 >= n) continue;
+            const uint32_t d = (key[j] >> shift) & mask;
+            const uint32_t p = S.start[d] + S.hist[warp][d] + rank[j];
+            S.keys[p] = key[j];
+            S.vals[p] = val[j];
+        }
+        __syncthreads();
+    }
+}
+
+// Compaction of the visible items and their depth sort.
+__global__ void __launch_bounds__(kOneThreads) k_small_depth_sort(const uint32_t *__restrict__ cnt,
+                                                                  const uint32_t *__restrict__ zkey, uint32_t n,
+                                                                  uint32_t *__restrict__ szkey,
+                                                                  uint32_t *__restrict__ sgid,
+                                                                  uint32_t *__restrict__ inv, uint32_t *d_m) {
+    pdl_enter();
+    extern __shared__ uint4 s_one[];
+    OneSmem &S = *reinterpret_cast<OneSmem *>(s_one);
+    const int tid = threadIdx.x;
+    const uint32_t per = (n + kOneThreads - 1) / kOneThreads, first = tid * per;
+    bool vis[kOneItems];
+    uint32_t z[kOneItems], mine = 0;
+#pragma unroll
+    for (int j = 0; j < kOneItems; j++) {
+        const uint32_t i = first + j;
+        const bool have = (uint32_t)j < per && i < n;
+        vis[j] = have && cnt[i] > 0u;
+        z[j] = have ? zkey[i] : 0u;  // (not written for invisible items, and not used then)
+        if (have && !vis[j]) inv[i] = 0xffffffffu;
+        mine += vis[j] ? 1u : 0u;
+    }
+    uint32_t M;
+    uint32_t off = block_excl_scan(mine, S.scan, &M);
+#pragma unroll
+    for (int j = 0; j < kOneItems; j++)
+        if (vis[j]) {
+            S.keys[off] = z[j];
+            S.vals[off++] = (uint16_t)(first + j);
+        }
+    __syncthreads();
+    one_cta_sort(S, M, 31);
+    for (uint32_t p = tid; p < M; p += kOneThreads) {
+        const uint32_t g = S.vals[p];
+        szkey[p] = S.keys[p];
+        sgid[p] = g;
+        inv[g] = p;
+    }
+    if (tid == 0) *d_m = M;
+}
+
+// Scan of the visible items' tile counts: first pair position per item, the
+// pair count K and the overflow flag, the first item of every expansion
+// chunk (of kEmitChunkSmall), and the tile ranges zeroed.
+__global__ void __launch_bounds__(kOneThreads) k_small_count(const uint32_t *__restrict__ vis_cnt, const uint32_t *d_m,
+                                                             uint32_t *__restrict__ vis_off,
+                                                             uint32_t *__restrict__ chunk_start, uint32_t capacity,
+                                                             uint32_t *d_k, uint32_t *overflow,
+                                                             uint32_t *__restrict__ ranges, uint32_t n_ranges) {
+    pdl_enter();
+    __shared__ uint32_t smem[33];
+    const int tid = threadIdx.x;
+    for (uint32_t i = tid; i < n_ranges; i += kOneThreads) ranges[i] = 0u;
+    const uint32_t M = *d_m, per = (M + kOneThreads - 1) / kOneThreads, first = tid * per;
+    uint32_t v[kOneItems], sum = 0;
+#pragma unroll
+    for (int j = 0; j < kOneItems; j++) {
+        v[j] = (uint32_t)j < per && first + j < M ? vis_cnt[first + j] : 0u;
+        sum += v[j];
+    }
+    uint32_t K;
+    uint32_t off = block_excl_scan(sum, smem, &K);
+#pragma unroll
+    for (int j = 0; j < kOneItems; j++) {
+        if ((uint32_t)j >= per || first + j >= M) break;
+        vis_off[first + j] = off;
+        const uint32_t end = min(off + v[j], capacity);
+        for (uint32_t c = (off + kEmitChunkSmall - 1) / kEmitChunkSmall; v[j] > 0u && c * kEmitChunkSmall < end; c++)
+            chunk_start[c] = first + j;
+        off += v[j];
+    }
+    if (tid == 0) {
+        *d_k = K;
+        if (K > capacity) *overflow = 1u;
+    }
+}
+
+// Tile sort of the K pairs, the tiles' ranges (zeroed before) and, with
+// `order`, the compositor's launch order (walk zeroed too).
+__global__ void __launch_bounds__(kOneThreads) k_small_tile_sort(const uint32_t *__restrict__ keys,
+                                                                 const uint32_t *__restrict__ vals,
+                                                                 uint32_t *__restrict__ vals_out, const uint32_t *d_k,
+                                                                 uint32_t capacity, int bits,
+                                                                 uint2 *__restrict__ ranges, uint32_t n_tiles,
+                                                                 uint32_t *__restrict__ order,
+                                                                 uint32_t *__restrict__ walk) {
+    pdl_enter();
+    extern __shared__ uint4 s_one[];
+    OneSmem &S = *reinterpret_cast<OneSmem *>(s_one);
+    const int tid = threadIdx.x;
+    const uint32_t K = min(*d_k, capacity);
+    if (order && walk)
+        for (uint32_t t = tid; t < n_tiles; t += kOneThreads) walk[t] = 0u;
+    for (uint32_t p = tid; p < K; p += kOneThreads) {
+        S.keys[p] = keys[p];
+        S.vals[p] = (uint16_t)vals[p];
+    }
+    __syncthreads();
+    one_cta_sort(S, K, bits);
+    for (uint32_t p = tid; p < K; p += kOneThreads) {
+        const uint32_t t = S.keys[p];
+        vals_out[p] = S.vals[p];
+        if (p == 0 || S.keys[p - 1] != t) ranges[t].x = p;
+        if (p + 1 == K || S.keys[p + 1] != t) ranges[t].y = p + 1;
+    }
+    if (order) {
+        __syncthreads();  // the ranges, read by this CTA
+        tile_order<1>(0, ranges, nullptr, n_tiles, order);
+    }
+}
+
+}  // namespace
+
+cudaError_t set_small_frame_smem() {
+    cudaError_t e = cudaFuncSetAttribute(k_small_depth_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(OneSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_small_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OneSmem));
+    return e;
+}
+
+size_t small_emit_chunks(uint64_t n_items, uint64_t tiles, uint32_t capacity) {
+    return (size_t)(std::min<uint64_t>(n_items * tiles, capacity) / kEmitChunkSmall + 2);
+}
+
+void small_depth_sort(const Params &p, cudaStream_t s) {
+    note_launch();
+    pdl_launch(k_small_depth_sort, 1, kOneThreads, sizeof(OneSmem), s, p.item_cnt, p.item_zkey, p.n_items, p.szkey,
+               p.sgid, p.inv, &p.counters[0]);
+}
+
+void small_count_pairs(const Params &p, cudaStream_t s) {
+    note_launch();
+    pdl_launch(k_small_count, 1, kOneThreads, 0, s, p.vis_cnt, (const uint32_t *)&p.counters[0], p.vis_off,
+               p.chunk_start, p.pair_capacity, &p.counters[1], &p.counters[2], reinterpret_cast<uint32_t *>(p.ranges),
+               2 * p.total_tiles);
+}
+
+void small_emit_pairs(const Params &p, void *temp, bool count_digits, cudaStream_t s) {
+    TempLayout t = temp_layout(temp);
+    // the general tile sort counts its first digits in the expansion
+    const int sort_items = p.pair_capacity <= kSmallSort ? kSmallItems : kSortItems;
+    const int sort_G = sort_blocks(p.pair_capacity, kSortThreads * sort_items);
+    if (count_digits) cudaMemsetAsync(t.hist, 0, sizeof(uint32_t) * kRadix * sort_G, s);
+    const uint32_t grid = std::min(std::max((p.pair_capacity + kEmitChunkSmall - 1) / kEmitChunkSmall, 1u),
+                                   (uint32_t)(8 * device_sm_count()));
+    note_launch();
+    pdl_launch(k_expand_pairs<kEmitChunkSmall>, grid, kEmitThreads, 0, s, p.vis_off, p.vis_cnt, p.chunk_start, p.rect,
+               p.rowtab, p.ell, p.tile_w, p.tile_h, p.vis_tile, p.vis_stride, p.views, p.n_views, &p.counters[0],
+               &p.counters[1], p.pair_capacity, p.pair_keys, p.pair_vals, count_digits ? t.hist : nullptr, sort_G,
+               (uint32_t)(kSortThreads * sort_items));
+}
+
+void small_tile_sort(const Params &p, uint32_t *vals_out, int bits, cudaStream_t s) {
+    const bool order = p.total_tiles <= kSmallOrderTiles;
+    note_launch();
+    pdl_launch(k_small_tile_sort, 1, kOneThreads, sizeof(OneSmem), s, p.pair_keys, p.pair_vals, vals_out,
+               (const uint32_t *)&p.counters[1], p.pair_capacity, bits, p.ranges, p.total_tiles,
+               order ? p.tile_order : nullptr, p.tile_walk);
+    if (!order) launch_tile_order(p, s);
 }
 
 void launch_tile_order(const Params &p, cudaStream_t s) {
