@@ -10,6 +10,7 @@
 // D += z alpha T, O += alpha T.  Every pixel's arithmetic is the same
 // expression whatever the tile and block shapes, so images are bit-identical
 // across them.
+#include <algorithm>
 #include <climits>
 
 #include "raster_fwd.cuh"
@@ -80,13 +81,31 @@ static Params with_shape(const Params &p, const WarpShape &w) {
     return q;
 }
 
+// One pixel per lane: where four would not fill the SMs (warp_shape gives
+// two), and the lists are short.  With long lists the issue slots bound the
+// pass, the sooner the more blocks the SMs have; with hardly any entries the
+// blocks themselves do.  Measured with two / one pixel per lane, by items per
+// block of 128 pixels, at 16 blocks per SM (641x479): 8: 23 / 20 us, 104: 95 /
+// 84, 416: 54 / 56; at 24 (1242x375): 16: 47 / 43, 69: 122 / 93, 137: 67 / 70,
+// 275: 71 / 80; at 46 (1000x900): 3: 25 / 29, 8: 43 / 41, 36: 86 / 78, 71: 78
+// / 95.  The line lies below the smallest loss: where few entries stop the
+// pixels, more items would still gain (four 640x480 views, 60 blocks per SM,
+// 110 items per block: 186 / 156), but their number does not tell.
+static bool one_pixel(const Params &p) {
+    const int64_t blocks = (int64_t)p.total_tiles * p.tile_w * p.tile_h / 128, sms = device_sm_count();
+    const int64_t items = p.n_items, full = 32 * sms;
+    return items >= 8 * blocks && items * std::max(blocks, full) <= 96 * blocks * full;
+}
+
 void launch_composite(const Params &p, cudaStream_t s) {
     if (p.total_tiles == 0) return;
     if (p.n_feat > 0) return launch_composite_feat(p, s);
-    const WarpShape w = warp_shape(p, kFwdWide, INT_MAX);
+    WarpShape w = warp_shape(p, kFwdWide, INT_MAX);
+    if (w.px == 2 && one_pixel(p)) w = WarpShape{1, 3, (uint32_t)(p.tile_w * p.tile_h / 32)};
     const Params q = with_shape(p, w);
     note_launch();
-    if (w.px == 4) pdl_launch(k_composite<4, 0>, p.total_tiles * w.blocks, 32, 0, s, q);
+    if (w.px == 1) pdl_launch(k_composite1<kFwdUnroll1>, p.total_tiles * w.blocks, 32, 0, s, q);
+    else if (w.px == 4) pdl_launch(k_composite<4, 0>, p.total_tiles * w.blocks, 32, 0, s, q);
     else pdl_launch(k_composite<2, 0>, p.total_tiles * w.blocks, 32, 0, s, q);
 }
 

@@ -82,6 +82,36 @@ struct Staged {
     float4 d[kStagedPlaces];  // (g, g, b, b)
     float2 e[kStagedPlaces];  // (z, z)
     uint32_t m[kStagedPlaces];
+
+    __device__ __forceinline__ void put(int k, const float4 &g, const float2 &q, const float4 &col, uint32_t pos,
+                                        uint32_t rec) {
+        a[k] = make_float4(g.x, g.z, g.w, __uint_as_float(pos));
+        b[k] = make_float4(g.y, g.y, q.x, q.x);
+        c[k] = make_float4(-q.y, -q.y, col.x, col.x);
+        d[k] = make_float4(col.y, col.y, col.z, col.z);
+        e[k] = make_float2(col.w, col.w);
+        m[k] = rec;
+    }
+};
+
+// The hits for one pixel per lane, whose packed arithmetic takes two
+// neighbouring entries.
+struct StagedEntries {
+    float u[kStagedPlaces], v[kStagedPlaces], a[kStagedPlaces], b[kStagedPlaces], c[kStagedPlaces];
+    float no[kStagedPlaces];       // -o~
+    uint32_t pos[kStagedPlaces];   // list position | flags
+    float4 col[kStagedPlaces];     // (r, g, b, z)
+
+    __device__ __forceinline__ void put(int k, const float4 &g, const float2 &q, const float4 &cl, uint32_t p, uint32_t) {
+        u[k] = g.x;
+        v[k] = g.y;
+        a[k] = g.z;
+        b[k] = g.w;
+        c[k] = q.x;
+        no[k] = -q.y;
+        pos[k] = p;
+        col[k] = cl;
+    }
 };
 
 // 32 records on their way to shared memory, one per lane
@@ -110,8 +140,8 @@ __device__ __forceinline__ void wait_records() { asm volatile("cp.async.wait_all
 // record's list position.  The places up to the next multiple of U get an
 // entry that blends nowhere.
 // items (optional): the hits' values of `item`, in their places.
-template <int U>
-__device__ __forceinline__ int stage_hits(const RawRecords &raw, Staged &S, bool have, uint32_t m, uint32_t pos,
+template <int U, class Stage>
+__device__ __forceinline__ int stage_hits(const RawRecords &raw, Stage &S, bool have, uint32_t m, uint32_t pos,
                                           const BlockGeom &G, int lane, uint32_t item = 0,
                                           uint32_t *items = nullptr) {
     bool hit = false;
@@ -129,22 +159,13 @@ __device__ __forceinline__ int stage_hits(const RawRecords &raw, Staged &S, bool
         const float s = fabsf(a.x) + fabsf(a.y) + fabsf(a.z) + fabsf(a.w) + fabsf(b.x) + fabsf(b.y) + fabsf(c.x) +
                         fabsf(c.y) + fabsf(c.z) + fabsf(c.w);
         pos |= (s < 1e30f ? 0u : kOddEntry) | (b.y <= kUncappedOpacity ? 0u : kCappedEntry);
-        S.a[k] = make_float4(a.x, a.z, a.w, __uint_as_float(pos));
-        S.b[k] = make_float4(a.y, a.y, b.x, b.x);
-        S.c[k] = make_float4(-b.y, -b.y, c.x, c.x);
-        S.d[k] = make_float4(c.y, c.y, c.z, c.z);
-        S.e[k] = make_float2(c.w, c.w);
-        S.m[k] = m;
+        S.put(k, a, b, c, pos, m);
         if (items) items[k] = item;
     }
     const int hits = __popc(mask);
     if (U > 1 && lane < (U - hits % U) % U) {
-        const int k = hits + lane;
-        S.a[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        S.b[k] = make_float4(0.f, 0.f, -kMinRowCoef, -kMinRowCoef);
-        S.c[k] = S.d[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        S.e[k] = make_float2(0.f, 0.f);
-        S.m[k] = 0u;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        S.put(hits + lane, zero, make_float2(-kMinRowCoef, 0.f), zero, 0u, 0u);
     }
     __syncwarp();
     return hits;

@@ -15,11 +15,15 @@ constexpr int kFwdUnroll = 4;
 // without spills (16 warps of 128 registers against 20 of 96: 280 and 310 us
 // on those views, 193 and 195 us on the 1.5M-Gaussian 1920x1280 frame).
 constexpr int kFwdWarps4 = 16, kFwdWarps2 = 20;
-// Blocks of 128 pixels per SM from which a lane takes four pixels and not
-// two: below it the longest walk bounds the pass and two pixels per lane
-// shorten it (9,100 blocks: 186 us with two, 280 us with four); above it the
-// issue slots do (19,200 blocks: 243 and 193 us).
+// Blocks of 128 pixels per SM from which a lane takes four pixels: below it
+// the longest walk bounds the pass and fewer pixels per lane shorten it
+// (four 640x480 views of 250k Gaussians, 9,100 blocks: 280 us with four, 186
+// us with two, 156 us with one); above it the issue slots do (1920x1280,
+// 19,200 blocks: 193, 243 and 313 us).
 constexpr int kFwdWide = 64;
+// With one pixel per lane (four entries together: 156 us on those views,
+// eight 164 us).
+constexpr int kFwdWarps1 = 24, kFwdUnroll1 = 4;
 // With extra channels: two pixels per lane (their sums fill the registers).
 // The longest walk bounds the pass here too (23 channels, 1242x375, 200k
 // Gaussians: 330 us with two entries together, 282 us with four).
@@ -317,6 +321,115 @@ __global__ void __launch_bounds__(32, NG > 0 ? kFwdWarpsFeat : PX == 4 ? kFwdWar
 #pragma unroll
         for (int p = 1; p < PX; p++) w = max(w, last[p]);
         w = __reduce_max_sync(0xffffffffu, w);
+        if (lane == 0 && w) atomicMax(&P.tile_walk[G.tile], w);
+    }
+}
+
+// The compositor with one pixel per lane: a block of 32 pixels has fewer
+// hits and its walk is the shortest, which frames need whose longest walks
+// bound the pass.  The packed arithmetic takes two neighbouring entries of
+// the pixel instead of two pixels: the same operations per pixel and entry,
+// half the issue slots, and nothing staged twice (961x641 with 300k
+// Gaussians: 104 us with two pixels per lane, 80 us with one).
+template <int U>
+__global__ void __launch_bounds__(32, kFwdWarps1) k_composite1(Params P) {
+    pdl_enter();
+    static_assert(U % 4 == 0 && kStagedPlaces % U == 0, "whole groups of four entries");
+    __shared__ RawRecords raw;
+    __shared__ __align__(16) StagedEntries S;
+    const int lane = threadIdx.x;
+    const BlockGeom G = block_geom<1>(P);
+    const ViewDesc &V = *G.V;
+    const uint2 r = G.r;
+    const uint32_t len = r.y - r.x;
+    const bool inside = G.px < V.W && G.py0 < V.H;
+    const float2 fx2 = make_float2((float)G.px + 0.5f, (float)G.px + 0.5f);
+    bool done = !inside;
+    float fy = done ? kFarRow : (float)G.py0 + 0.5f;  // (far away once done: blends nothing)
+    float T[1] = {1.0f}, C0[1] = {-0.0f}, C1[1] = {-0.0f}, C2[1] = {-0.0f}, D[1] = {-0.0f}, O[1] = {-0.0f};  // sums negated
+    uint32_t last[1] = {inside ? len : 0u};
+    uint32_t m0 = lane < len ? P.pair_vals[r.x + lane] : kNoRecord;
+    fetch_record(P, raw, m0, lane);
+    uint32_t m1 = lane + 32u < len ? P.pair_vals[r.x + 32u + lane] : kNoRecord;
+    bool finished = __all_sync(0xffffffffu, done);
+    for (uint32_t base = 0; base < len && !finished; base += 32) {
+        wait_records();
+        const int hits = stage_hits<U>(raw, S, m0 != kNoRecord, m0, base + lane, G, lane);
+        m0 = m1;
+        fetch_record(P, raw, m0, lane);
+        m1 = base + 64u + lane < len ? P.pair_vals[r.x + base + 64u + lane] : kNoRecord;
+        for (int k = 0; k < hits; k += U) {
+            const float2 fy2 = make_float2(fy, fy);
+            float na[U];  // -alpha, -0 where the pixel does not blend
+            uint32_t flags = 0;
+#pragma unroll
+            for (int g = 0; g < U / 4; g++) {
+                auto four = [&](const float *f) { return reinterpret_cast<const float4 *>(f + k)[g]; };
+                const float4 u = four(S.u), v = four(S.v), a = four(S.a), b = four(S.b), c = four(S.c), no = four(S.no);
+                const uint4 p = reinterpret_cast<const uint4 *>(S.pos + k)[g];
+                flags |= p.x | p.y | p.z | p.w;
+                auto two = [&](float2 u2, float2 v2, float2 a2, float2 b2, float2 c2, float2 no2, float *out) {
+                    const float2 dx = sub2(fx2, u2), dy = sub2(fy2, v2);
+                    const float2 e = falloff_exp2_x2(mul2(mul2(a2, dx), dx), mul2(b2, dx), c2, dy);
+                    const float2 nr = mul2(no2, make_float2(ex2_approx(e.x), ex2_approx(e.y)));
+                    out[0] = nr.x <= -kAlphaMin ? nr.x : -0.0f;
+                    out[1] = nr.y <= -kAlphaMin ? nr.y : -0.0f;
+                };
+                two(make_float2(u.x, u.y), make_float2(v.x, v.y), make_float2(a.x, a.y), make_float2(b.x, b.y),
+                    make_float2(c.x, c.y), make_float2(no.x, no.y), na + 4 * g);
+                two(make_float2(u.z, u.w), make_float2(v.z, v.w), make_float2(a.z, a.w), make_float2(b.z, b.w),
+                    make_float2(c.z, c.w), make_float2(no.z, no.w), na + 4 * g + 2);
+            }
+            if (flags > kPosMask) {  // o~ may exceed the cap (one that cannot is left as it is)
+#pragma unroll
+                for (int u = 0; u < U; u++) na[u] = fmaxf(na[u], -kAlphaCap);
+            }
+            float nw[U], t = T[0];
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                nw[u] = __fmul_rn(na[u], t);
+                t = __fadd_rn(t, nw[u]);
+            }
+            // T only falls, so the pixel stops in these entries exactly if its
+            // T after the last of them is below the stop
+            const bool any_stop = __any_sync(0xffffffffu, t < kTStop);
+            if (any_stop && t < kTStop) {  // no part from the entry that would stop it on
+                t = T[0];
+#pragma unroll
+                for (int u = 0; u < U; u++) {
+                    if (!done && __fadd_rn(t, nw[u]) < kTStop) {
+                        done = true;
+                        last[0] = S.pos[k + u] & kPosMask;
+                        fy = kFarRow;
+                    }
+                    if (done) nw[u] = -0.0f;
+                    t = __fadd_rn(t, nw[u]);
+                }
+            }
+            T[0] = t;
+            const bool odd = flags & kOddEntry;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const float4 col = S.col[k + u];
+                if (odd && nw[u] == 0.0f) continue;  // non-finite terms: a zero weight must not meet them
+                C0[0] = __fmaf_rn(col.x, nw[u], C0[0]);
+                C1[0] = __fmaf_rn(col.y, nw[u], C1[0]);
+                C2[0] = __fmaf_rn(col.z, nw[u], C2[0]);
+                D[0] = __fmaf_rn(col.w, nw[u], D[0]);
+                O[0] = __fadd_rn(O[0], nw[u]);
+            }
+            if (any_stop && __all_sync(0xffffffffu, done)) {
+                finished = true;
+                break;
+            }
+        }
+        __syncwarp();  // the next group restages
+    }
+    wait_records();  // a copy may still be under way when the walk ended early
+    C0[0] = -C0[0]; C1[0] = -C1[0]; C2[0] = -C2[0]; D[0] = -D[0]; O[0] = -O[0];
+    composite_epilogue<1>(P, V, G, T, C0, C1, C2, D, O, last);
+    if (P.tile_walk) {
+        const uint32_t w = __reduce_max_sync(0xffffffffu, last[0]);
         if (lane == 0 && w) atomicMax(&P.tile_walk[G.tile], w);
     }
 }

@@ -62,6 +62,44 @@ def test_blocks_of_every_width_agree(cfg, aux):
         assert torch.linalg.norm(gn[k].double() - want) <= 1e-4 * torch.linalg.norm(want), k
 
 
+@pytest.mark.parametrize("size", [(97, 61), (161, 37)])
+@pytest.mark.parametrize("cfg", T.CONFIGS)
+def test_one_and_two_pixels_per_lane_agree(cfg, size):
+    """The compositor's pixels per lane in a small frame follow from the
+    number of items per block of pixels: Gaussians too faint to be seen take
+    the same view through one pixel per lane (36 items per block) and two
+    (about 5 and 300), with the same images bit for bit, gradients that agree
+    (equal sums in another order: 1e-4 of the norm) and infinite colours in
+    the same pixels."""
+    scene = synth.make_plain_scene(seed=4, n=300, sh_degree=1, log_scale_mean=-2.3)
+    scene["opacity"][::7] = 1.0
+    cam = synth.plain_camera(*size, t=0.4, bg=(0.2, 0.1, 0.3))
+    tx, ty = R.tiles_of(cam, cfg[:2])
+    blocks = tx * ty * cfg[0] * cfg[1] / 128
+    r = R.Renderer(tile=cfg[:2], pixels_per_thread=cfg[2])
+    d = _weights(cam, True)
+    for bad in (False, True):
+        if bad:
+            scene["sh"][int(np.argmax(scene["opacity"]))] = np.inf
+        ref = None
+        for per_block in (3, 36, 300):
+            n = max(300, int(per_block * blocks)) - 300
+            part = {k: np.concatenate([v, np.repeat(v[:1], n, axis=0)]) for k, v in scene.items()}
+            part["opacity"][300:] = 1e-4
+            fr = R.Frame()
+            st = R.scene_to_device(part)
+            out = r.forward(st, [cam], frame=fr)[0]
+            cur = [out[k].clone() for k in ("rgb", "depth", "alpha")]
+            if not bad:
+                cur.append(r.backward(st, [cam], fr, [d])["opacity"][:300].clone())
+            if ref is None:
+                ref = cur
+            for x, y in zip(ref[:3], cur[:3]):
+                assert torch.equal(torch.nan_to_num(x, nan=7.0), torch.nan_to_num(y, nan=7.0)), (bad, per_block)
+            for x, y in zip(ref[3:], cur[3:]):
+                assert torch.linalg.norm(x - y) <= 1e-4 * torch.linalg.norm(x), per_block
+
+
 @pytest.mark.parametrize("repeat", [False, True])
 @pytest.mark.parametrize("cfg", [(16, 16, 1), (16, 8, 1), (32, 32, 4)])
 def test_non_finite_values_stay_where_they_blend(cfg, repeat):
