@@ -5,6 +5,8 @@
 // Sec. 3.2, Eq. 6-8; the flow shift of Sec. 3.4).  Visibility comes from
 // inv[]; the projection is recomputed for its intermediate terms only, so
 // this file may contract a*b+c into fused multiply-adds.
+#include <algorithm>
+
 #include "preprocess_common.cuh"
 
 namespace pvg {
@@ -265,76 +267,138 @@ __device__ __forceinline__ bool item_adjoint(const Params &P, const ViewDesc &V,
 // the warp), accumulates the item adjoints over those views -- the 17 small
 // gradients in registers, the SH-coefficient gradients in a column of
 // shared memory -- and writes every gradient entry once: no atomics and no
-// zeroing pass.  Warps take 32 consecutive Gaussians at a time.
+// zeroing pass.  A warp takes 32 PER consecutive Gaussians; with PER > 1 it
+// works on them 32 at a time in the order of their numbers of views, so that
+// its lanes walk about as many (as they come, 14 of 32 lanes are active: 1M
+// Gaussians in 12 views 870 us with PER = 1, 747 with 2, 792 with 4, 893 with
+// 8, whose last chunks run alone; all lanes at the same view, the next one's
+// gradients on their way: 960 us).
 constexpr int kViewsThreads = 128;
 
-template <int D>
+template <int D, int PER>
 __global__ void __launch_bounds__(kViewsThreads) k_preprocess_bwd_views(Params P) {
     pdl_enter();
     constexpr int K = (D + 1) * (D + 1);
+    constexpr int kViewsChunk = 32 * PER;
+    constexpr uint32_t kWarps = kViewsThreads / 32;
     extern __shared__ float s_sh[];  // [3 K][kViewsThreads]
-    const int tid = threadIdx.x;
+    __shared__ unsigned long long s_mask[kWarps][kViewsChunk];  // the first 64 views that see a Gaussian
+    __shared__ uint8_t s_order[kWarps][kViewsChunk];
+    __shared__ uint32_t s_first[kWarps][65];  // per number of views: Gaussians with more
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const ViewDesc &V0 = P.views[0];  // every view renders the same scene (gradient pointers too)
     const uint32_t n = V0.n;
     float *col = V0.g_sh ? s_sh + tid : nullptr;
-    // a warp's first 32 Gaussians by its index, the next ones from a ticket
+    // a warp's first chunk by its index, the next ones from a ticket
     // (counters[3], reset by the adjoint's first kernel): the Gaussians seen
     // by more views cost more, and the warps done first take more
-    constexpr uint32_t kWarps = kViewsThreads / 32;
-    const int lane = tid & 31;
-    uint32_t w = blockIdx.x * kWarps + (uint32_t)(tid >> 5);
-    for (;;) {
-        const uint32_t i = w * 32u + (uint32_t)lane;
-        if (w * 32u >= n) break;
+    uint32_t c = blockIdx.x * kWarps + (uint32_t)warp;
+    const uint32_t n_chunks = (n + kViewsChunk - 1) / kViewsChunk;
+    while (c < n_chunks) {
+        const uint32_t base = c * kViewsChunk;
         {
             uint32_t t = 0;
             if (lane == 0) t = atomicAdd(&P.counters[3], 1u);
-            w = __shfl_sync(0xffffffffu, t, 0) + gridDim.x * kWarps;
+            c = __shfl_sync(0xffffffffu, t, 0) + gridDim.x * kWarps;
         }
-        if (i >= n) continue;
-        SmallGrads acc = SmallGrads{};
-        if (col)
-#pragma unroll
-            for (int c = 0; c < 3 * K; c++) col[c * kViewsThreads] = 0.f;
-        for (int v0 = 0; v0 < P.n_views; v0 += 64) {
+        // the views v0 .. v0 + 63 that see Gaussian i
+        auto views_of = [&](uint32_t i, int v0) {
             const int vn = min(64, P.n_views - v0);
             unsigned long long mask = 0ull;
+#pragma unroll 4
             for (int v = 0; v < vn; v++)
                 if (P.inv[P.views[v0 + v].item_base + i] != 0xffffffffu) mask |= 1ull << v;
-            while (mask) {
-                const int v = __ffsll((long long)mask) - 1;
-                mask &= mask - 1ull;
-                const ViewDesc &V = P.views[v0 + v];
-                SmallGrads q;
-                if (!item_adjoint<D>(P, V, i, P.inv[V.item_base + i], false, q, col, kViewsThreads)) continue;
+            return mask;
+        };
+        if constexpr (PER > 1) {
+            // counting sort by the number of (the first 64) views, most first
+            for (int b = lane; b < 65; b += 32) s_first[warp][b] = 0u;
+            __syncwarp();
+            unsigned long long mine[PER];
+#pragma unroll
+            for (int q = 0; q < PER; q++) {
+                const uint32_t i = base + 32 * q + lane;
+                mine[q] = i < n ? views_of(i, 0) : 0ull;
+                s_mask[warp][32 * q + lane] = mine[q];
+                atomicAdd(&s_first[warp][64 - __popcll(mine[q])], 1u);
+            }
+            __syncwarp();
+            {
+                uint32_t cnt[3], sum = 0;  // a lane's bins 3 lane .. 3 lane + 2 (65 bins)
 #pragma unroll
                 for (int k = 0; k < 3; k++) {
-                    acc.mu[k] += q.mu[k];
-                    acc.vel[k] += q.vel[k];
-                    acc.scale[k] += q.scale[k];
+                    cnt[k] = 3 * lane + k < 65 ? s_first[warp][3 * lane + k] : 0u;
+                    sum += cnt[k];
                 }
+                uint32_t before = sum;
 #pragma unroll
-                for (int k = 0; k < 4; k++) acc.quat[k] += q.quat[k];
-                acc.tau += q.tau;
-                acc.beta += q.beta;
-                acc.period += q.period;
-                acc.opac += q.opac;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t v = __shfl_up_sync(0xffffffffu, before, o);
+                    if (lane >= o) before += v;
+                }
+                before -= sum;
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < 3; k++)
+                    if (3 * lane + k < 65) {
+                        s_first[warp][3 * lane + k] = before;
+                        before += cnt[k];
+                    }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < PER; q++)
+                s_order[warp][atomicAdd(&s_first[warp][64 - __popcll(mine[q])], 1u)] = (uint8_t)(32 * q + lane);
+            __syncwarp();
+        }
+        for (int g = 0; g < PER; g++) {
+            const uint32_t at = PER > 1 ? s_order[warp][32 * g + lane] : (uint32_t)lane, i = base + at;
+            if (i >= n) continue;
+            SmallGrads acc = SmallGrads{};
+            if (col)
+#pragma unroll
+                for (int e = 0; e < 3 * K; e++) col[e * kViewsThreads] = 0.f;
+            unsigned long long mask = PER > 1 ? s_mask[warp][at] : views_of(i, 0);
+            for (int v0 = 0;;) {
+                while (mask) {
+                    const int v = __ffsll((long long)mask) - 1;
+                    mask &= mask - 1ull;
+                    const ViewDesc &V = P.views[v0 + v];
+                    SmallGrads q;
+                    if (!item_adjoint<D>(P, V, i, P.inv[V.item_base + i], false, q, col, kViewsThreads)) continue;
+#pragma unroll
+                    for (int k = 0; k < 3; k++) {
+                        acc.mu[k] += q.mu[k];
+                        acc.vel[k] += q.vel[k];
+                        acc.scale[k] += q.scale[k];
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; k++) acc.quat[k] += q.quat[k];
+                    acc.tau += q.tau;
+                    acc.beta += q.beta;
+                    acc.period += q.period;
+                    acc.opac += q.opac;
+                }
+                v0 += 64;
+                if (v0 >= P.n_views) break;
+                mask = views_of(i, v0);
+            }
+            if (V0.g_mu) for (int k = 0; k < 3; k++) V0.g_mu[3 * (size_t)i + k] = acc.mu[k];
+            if (V0.g_vel) for (int k = 0; k < 3; k++) V0.g_vel[3 * (size_t)i + k] = acc.vel[k];
+            if (V0.g_scale) for (int k = 0; k < 3; k++) V0.g_scale[3 * (size_t)i + k] = acc.scale[k];
+            if (V0.g_quat) for (int k = 0; k < 4; k++) V0.g_quat[4 * (size_t)i + k] = acc.quat[k];
+            if (V0.g_tau) V0.g_tau[i] = acc.tau;
+            if (V0.g_beta) V0.g_beta[i] = acc.beta;
+            if (V0.g_period) V0.g_period[i] = acc.period;
+            if (V0.g_opac) V0.g_opac[i] = acc.opac;
+            if (col) {
+                float g4[3 * K];
+#pragma unroll
+                for (int e = 0; e < 3 * K; e++) g4[e] = col[e * kViewsThreads];
+                store_floats<3 * K>(V0.g_sh + (size_t)i * 3 * K, g4, aligned16(V0.g_sh));
             }
         }
-        if (V0.g_mu) for (int k = 0; k < 3; k++) V0.g_mu[3 * (size_t)i + k] = acc.mu[k];
-        if (V0.g_vel) for (int k = 0; k < 3; k++) V0.g_vel[3 * (size_t)i + k] = acc.vel[k];
-        if (V0.g_scale) for (int k = 0; k < 3; k++) V0.g_scale[3 * (size_t)i + k] = acc.scale[k];
-        if (V0.g_quat) for (int k = 0; k < 4; k++) V0.g_quat[4 * (size_t)i + k] = acc.quat[k];
-        if (V0.g_tau) V0.g_tau[i] = acc.tau;
-        if (V0.g_beta) V0.g_beta[i] = acc.beta;
-        if (V0.g_period) V0.g_period[i] = acc.period;
-        if (V0.g_opac) V0.g_opac[i] = acc.opac;
-        if (col) {
-            float g[3 * K];
-#pragma unroll
-            for (int c = 0; c < 3 * K; c++) g[c] = col[c * kViewsThreads];
-            store_floats<3 * K>(V0.g_sh + (size_t)i * 3 * K, g, aligned16(V0.g_sh));
-        }
+        __syncwarp();  // the next chunk's masks and order
     }
 }
 
@@ -503,21 +567,32 @@ __global__ void __launch_bounds__(256, 3) k_preprocess_bwd(Params P) {
 
 }  // namespace
 
+// Two Gaussians per lane, ordered, from two rounds of them for the resident
+// warps (four blocks per SM); with fewer the last round runs half empty (with
+// one / two, 12 views: 20k 50 / 76 us, 60k 72 / 93, 200k 201 / 218, 400k 385 /
+// 339, 1M 867 / 732; 2 views: 200k 54 / 59, 400k 98 / 95, 1M 217 / 196).
+template <int D>
+static void launch_views(const Params &p, uint32_t n, cudaStream_t s) {
+    constexpr uint32_t kWarps = kViewsThreads / 32;
+    const uint32_t sms = (uint32_t)device_sm_count();
+    const bool two = n >= 2u * 64u * 4u * kWarps * sms;
+    const uint32_t per = kWarps * (two ? 64u : 32u);
+    const uint32_t grid = std::max(1u, std::min((n + per - 1) / per, 16u * sms));
+    const size_t smem = sizeof(float) * 3 * (D + 1) * (D + 1) * kViewsThreads;
+    if (two) pdl_launch(k_preprocess_bwd_views<D, 2>, grid, kViewsThreads, smem, s, p);
+    else pdl_launch(k_preprocess_bwd_views<D, 1>, grid, kViewsThreads, smem, s, p);
+}
+
 void launch_preprocess_bwd(const Params &p, bool several_views, cudaStream_t s) {
     note_launch();
     if (several_views) {
         // the host copy of the views: every view has the scene's n items
         const uint32_t n = p.n_views > 0 ? p.n_items / (uint32_t)p.n_views : 0u;
-        uint32_t grid = (n + kViewsThreads - 1) / kViewsThreads;
-        const uint32_t cap = 16u * (uint32_t)device_sm_count();
-        if (grid > cap) grid = cap;
-        if (grid < 1) grid = 1;
-        const size_t smem = sizeof(float) * 3 * (p.sh_degree + 1) * (p.sh_degree + 1) * kViewsThreads;
         switch (p.sh_degree) {
-            case 0: pdl_launch(k_preprocess_bwd_views<0>, grid, kViewsThreads, smem, s, p); break;
-            case 1: pdl_launch(k_preprocess_bwd_views<1>, grid, kViewsThreads, smem, s, p); break;
-            case 2: pdl_launch(k_preprocess_bwd_views<2>, grid, kViewsThreads, smem, s, p); break;
-            default: pdl_launch(k_preprocess_bwd_views<3>, grid, kViewsThreads, smem, s, p); break;
+            case 0: launch_views<0>(p, n, s); break;
+            case 1: launch_views<1>(p, n, s); break;
+            case 2: launch_views<2>(p, n, s); break;
+            default: launch_views<3>(p, n, s); break;
         }
         return;
     }
