@@ -50,13 +50,35 @@ __global__ void k_feat_param_bwd(Params P) {
 
 }  // namespace
 
+// Four pixels per lane from kFeatBwdWide blocks of 128 pixels per SM, as far
+// as their output gradients fit the registers (32 channels); two below (23
+// channels, four / two: 1920x1280 with 1.5M Gaussians 2.16 / 3.17 ms,
+// 1242x800 with 100k 574 / 681 us, 1242x375 with 300k 1,006 / 746 us).
+constexpr int kFeatBwdWide = 40, kFeatBwdWideGroups = 8;
+
 void launch_composite_feat_bwd(const Params &p, cudaStream_t s) {
+    const int groups = (p.n_feat + 3) / 4, pixels = p.tile_w * p.tile_h;
+    const bool wide = groups <= kFeatBwdWideGroups && pixels >= 128 &&
+                      (int64_t)p.total_tiles * pixels / 128 >= (int64_t)kFeatBwdWide * device_sm_count();
     Params q = p;
-    q.block_shift = 3;
-    q.blocks_per_tile = (uint32_t)(p.tile_w * p.tile_h / 64);
+    q.block_shift = wide && p.tile_h < 16 ? 4 : 3;
+    q.blocks_per_tile = (uint32_t)(pixels / (wide ? 128 : 64));
     const uint32_t grid = p.total_tiles * q.blocks_per_tile;
     note_launch();
-    switch ((p.n_feat + 3) / 4) {
+    if (wide) {
+        switch (groups) {
+            case 1: pdl_launch(k_composite_bwd<4, true, 1>, grid, 32, 0, s, q); break;
+            case 2: pdl_launch(k_composite_bwd<4, true, 2>, grid, 32, 0, s, q); break;
+            case 3: pdl_launch(k_composite_bwd<4, true, 3>, grid, 32, 0, s, q); break;
+            case 4: pdl_launch(k_composite_bwd<4, true, 4>, grid, 32, 0, s, q); break;
+            case 5: pdl_launch(k_composite_bwd<4, true, 5>, grid, 32, 0, s, q); break;
+            case 6: pdl_launch(k_composite_bwd<4, true, 6>, grid, 32, 0, s, q); break;
+            case 7: pdl_launch(k_composite_bwd<4, true, 7>, grid, 32, 0, s, q); break;
+            default: pdl_launch(k_composite_bwd<4, true, 8>, grid, 32, 0, s, q); break;
+        }
+        return;
+    }
+    switch (groups) {
         case 1: pdl_launch(k_composite_bwd<2, true, 1>, grid, 32, 0, s, q); break;
         case 2: pdl_launch(k_composite_bwd<2, true, 2>, grid, 32, 0, s, q); break;
         case 3: pdl_launch(k_composite_bwd<2, true, 3>, grid, 32, 0, s, q); break;

@@ -168,3 +168,34 @@ def test_channels_keep_the_colour_pass_and_their_non_finite_values(mask, n_sem):
         assert 0 < int((weight > 0).sum()) < weight.numel()
         assert torch.equal(torch.isnan(feat[-1]), weight > 0)
         assert torch.isfinite(feat[:-1]).all()
+
+
+@pytest.mark.parametrize("mask,n_sem", [(abi.FEAT_RHO, 0), (abi.FEAT_SEM, 24), (7, 28), (7, 32)])
+@pytest.mark.parametrize("cfg", [(8, 8, 1), (16, 8, 1), (32, 32, 4)])
+def test_channel_blocks_of_every_width_agree(cfg, mask, n_sem):
+    """The channel passes' two and four pixels per lane (the view alone and
+    repeated; 32 and 36 channels keep two in the forward, 36 in both): the
+    same images bit for bit, gradients that add up (the tolerance above)."""
+    scene = synth.make_plain_scene(seed=4, n=300, sh_degree=1, log_scale_mean=-2.3)
+    st = R.scene_to_device(scene)
+    if n_sem:
+        st["sem"] = torch.tensor(synth.make_semantics(300, n_sem), device="cuda")
+    cam = synth.plain_camera(97, 61, t=0.4, bg=(0.2, 0.1, 0.3))
+    r = R.Renderer(tile=cfg[:2], pixels_per_thread=cfg[2])
+    one, many = R.Frame(), R.Frame()
+    ref = r.forward(st, [cam], frame=one, features=mask)[0]
+    d = _weights(cam, True)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(8)
+    d["feat"] = torch.randn(*ref["feat"].shape, generator=g, device="cuda")
+    g1 = r.backward(st, [cam], one, [d])
+    cams = _views(cam, cfg)
+    outs = r.forward(st, cams, frame=many, features=mask)
+    gn = r.backward(st, cams, many, [d] * len(cams))
+    for v in (0, len(cams) // 2, len(cams) - 1):
+        for k in ("rgb", "depth", "alpha", "feat"):
+            assert torch.equal(outs[v][k], ref[k]), (v, k)
+    for k in [*R.PARAM_NAMES] + (["sem"] if n_sem else []):
+        want = g1[k].double() * len(cams)
+        assert torch.linalg.norm(want) > 0, k
+        assert torch.linalg.norm(gn[k].double() - want) <= 1e-4 * torch.linalg.norm(want), k
