@@ -52,8 +52,9 @@ __global__ void k_feat_param_bwd(Params P) {
 
 // Four pixels per lane from kFeatBwdWide blocks of 128 pixels per SM, as far
 // as their output gradients fit the registers (32 channels); two below (23
-// channels, four / two: 1920x1280 with 1.5M Gaussians 2.16 / 3.17 ms,
-// 1242x800 with 100k 574 / 681 us, 1242x375 with 300k 1,006 / 746 us).
+// channels, four / two, before the arithmetic on channels was packed by them:
+// 1920x1280 with 1.5M Gaussians 2.16 / 3.17 ms, 1242x800 with 100k 574 / 681
+// us, 1242x375 with 300k 1,006 / 746 us; since then 1.83 ms, 451 and 706 us).
 constexpr int kFeatBwdWide = 40, kFeatBwdWideGroups = 8;
 
 void launch_composite_feat_bwd(const Params &p, cudaStream_t s) {

@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kFwdWarpsFeat : PX == 4 ? kFwdWar
     constexpr uint32_t ALL = (1u << PX) - 1u;
     __shared__ RawRecords raw;
     __shared__ Staged S;
-    __shared__ StagedFeats<NG> F;
+    __shared__ StagedFeats<NG, true> F;
     const int lane = threadIdx.x;
     const BlockGeom G = block_geom<PX>(P);
     const ViewDesc &V = *G.V;
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kFwdWarpsFeat : PX == 4 ? kFwdWar
     far_rows();
     uint32_t m0 = lane < len ? P.pair_vals[r.x + lane] : kNoRecord;
     fetch_record(P, raw, m0, lane);
-    if constexpr (NG > 0) clear_feats<NG>(F, lane);
+    if constexpr (NG > 0) clear_feats(F, lane);
     uint32_t i0 = 0;  // the lane's Gaussian
     if constexpr (NG > 0) i0 = m0 != kNoRecord ? P.sgid[m0] - V.item_base : 0u;
     uint32_t m1 = lane + 32u < len ? P.pair_vals[r.x + 32u + lane] : kNoRecord;
