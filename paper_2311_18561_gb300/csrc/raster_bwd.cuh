@@ -27,7 +27,7 @@ struct BwdTune {
 // with four.  Two only for frames too small for four (1242x375: 178 us with
 // two, 133 us with four).
 constexpr int kBwdWide8 = 48, kBwdWide4 = 16;
-// With extra channels: two pixels per lane, and two entries' channel sums
+// With extra channels (two or four pixels per lane): two entries' channel sums
 // taken together (23 channels, 1242x375, 200k Gaussians: 723 us one by one,
 // 638 us by twos, 641 us by fours).
 constexpr int kBwdWarpsFeat = 8, kBwdUnrollFeat = 2;

@@ -173,34 +173,32 @@ __device__ __forceinline__ int stage_hits(const RawRecords &raw, Stage &S, bool 
     return hits;
 }
 
-// Extra channels of the staged entries, zeros beyond the call's channels; kTwice:
-// each value twice (operands of arithmetic on pairs of pixels).
-template <int NG, bool kTwice>
+// Extra channels of the staged entries, zeros beyond the call's channels.  The
+// arithmetic on channels is packed by pairs of channels, which needs no value
+// twice.
+template <int NG>
 struct StagedFeats {
-    alignas(16) typename std::conditional<kTwice, float2, float>::type f[kStagedPlaces][4 * NG];
+    alignas(16) float f[kStagedPlaces][4 * NG];
     uint32_t item[kStagedPlaces];  // Gaussian of the entry's scene
 };
-template <bool kTwice>
-struct StagedFeats<0, kTwice> {};
-
-__device__ __forceinline__ void put_value(float2 &f, float v) { f = make_float2(v, v); }
-__device__ __forceinline__ void put_value(float &f, float v) { f = v; }
+template <>
+struct StagedFeats<0> {};
 
 // Zeroes the channel values once: those beyond the call's channels stay zero.
-template <int NG, bool kTwice>
-__device__ __forceinline__ void clear_feats(StagedFeats<NG, kTwice> &F, int lane) {
-    for (int k = lane; k < kStagedPlaces * (kTwice ? 2 : 1) * NG; k += 32)
+template <int NG>
+__device__ __forceinline__ void clear_feats(StagedFeats<NG> &F, int lane) {
+    for (int k = lane; k < kStagedPlaces * NG; k += 32)
         reinterpret_cast<float4 *>(&F.f[0][0])[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // The channel values of the `hits` staged entries (their Gaussians in
 // F.item; places up to the next multiple of U zeroed): every semantic row by
 // the whole warp, all rows' copies in flight together and behind them v_bar
-// and rho by the entries' lanes; then one pass doubles the semantic values
-// (kTwice) and looks for those that are not finite.
+// and rho by the entries' lanes; then one pass looks for semantic values that
+// are not finite.
 // Entries with non-finite values are flagged in S.
-template <int NG, int U, bool kTwice>
-__device__ __forceinline__ void stage_feats(const Params &P, const ViewDesc &V, Staged &S, StagedFeats<NG, kTwice> &F,
+template <int NG, int U>
+__device__ __forceinline__ void stage_feats(const Params &P, const ViewDesc &V, Staged &S, StagedFeats<NG> &F,
                                             int hits, int lane) {
     const int places = (hits + U - 1) / U * U;
     const int c0 = ((P.feat_mask & kFeatVbar) ? 3 : 0) + ((P.feat_mask & kFeatRho) ? 1 : 0);
@@ -218,7 +216,7 @@ __device__ __forceinline__ void stage_feats(const Params &P, const ViewDesc &V, 
         float bad = 0.f;
         int c = 0;
         auto put = [&](float v) {
-            put_value(F.f[lane][c++], v);
+            F.f[lane][c++] = v;
             bad += fabsf(v);
         };
         if (P.feat_mask & kFeatVbar) {
@@ -232,17 +230,14 @@ __device__ __forceinline__ void stage_feats(const Params &P, const ViewDesc &V, 
         if (!(bad < 1e30f)) S.a[lane].w = __uint_as_float(__float_as_uint(S.a[lane].w) | kOddEntry);
     }
     for (int k = hits; k < places; k++)
-        for (int c = lane; c < 4 * NG; c += 32) put_value(F.f[k][c], 0.f);
+        for (int c = lane; c < 4 * NG; c += 32) F.f[k][c] = 0.f;
     if (n_sem) {
         wait_records();
         uint32_t bad = 0;  // entries with a non-finite value of this lane's class
         if (lane < n_sem)
 #pragma unroll 4
             for (int k = 0; k < hits; k++) {
-                auto &f = F.f[k][c0 + lane];
-                const float v = *reinterpret_cast<const float *>(&f);
-                if constexpr (kTwice) f.y = v;
-                bad |= fabsf(v) < 1e30f ? 0u : 1u << k;
+                bad |= fabsf(F.f[k][c0 + lane]) < 1e30f ? 0u : 1u << k;
             }
         bad = __reduce_or_sync(0xffffffffu, bad);
         if ((bad >> lane) & 1u) S.a[lane].w = __uint_as_float(__float_as_uint(S.a[lane].w) | kOddEntry);
