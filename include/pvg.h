@@ -207,7 +207,9 @@ typedef struct {
     int32_t pixels_per_thread; /* compositing pixels per thread (1, 2 or 4; 0 = 1).
                              * Supported (tile_w, tile_h, pixels_per_thread):
                              * (16,16,1|2|4) (8,8,1|2) (16,8,1|2) (32,8,1)
-                             * (32,16,1|2|4) (32,32,4) (16,32,4).  Images do not
+                             * (32,16,1|2|4) (32,32,4) (16,32,4).  Checked and kept
+                             * with the frame; the kernels choose their pixels
+                             * per lane by the frame's size.  Images do not
                              * depend on the choice (bit-identical). */
     int64_t pair_capacity;  /* pairs per frame when sync_sizes = 0 */
     float dilation;         /* EWA low-pass h in px^2 (default 0.3) */

@@ -11,7 +11,8 @@
 //   b  scan + emit          (tile, m) pairs in depth order, K
 //      radix sort           by tile id (ceil(log2 tiles) bits)
 //      k_ranges             [start, end) per tile
-//   c  k_composite          images + per-pixel T and last position
+//   c  k_composite          images + per-pixel T and stop position
+// (a frame of at most kSmallFrameItems items takes one CTA per sorting stage)
 // Backward: k_composite_bwd (image-space gradients per record) and
 // k_preprocess_bwd (parameter gradients).
 #include <algorithm>

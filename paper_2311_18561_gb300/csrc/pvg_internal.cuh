@@ -16,7 +16,7 @@
 //     vis_cnt[m] tiles of the rectangle that the footprint ellipse meets
 //   pairs     (tile, m) pairs sorted by (tile, depth, gid)             [K]
 //   ranges    [start, end) into the pairs per global tile             [tiles]
-//   pixels    final transmittance and last blended list position      [sum HW]
+//   pixels    final transmittance and stop position in the list       [sum HW]
 #pragma once
 #include <cstdint>
 #include <utility>
@@ -116,9 +116,9 @@ struct Params {
     uint32_t *pair_vals;     // [K]
     uint2 *ranges;           // [total_tiles]
     uint32_t *tile_order;    // [total_tiles] tiles by decreasing list length (compositor launch order)
-    uint32_t *tile_walk;     // [total_tiles] forward: largest pixel_last of the tile (the adjoint's walk)
+    uint32_t *tile_walk;     // [total_tiles] forward: largest pix_last of the tile (the adjoint's walk)
     float *pix_T;            // [sum HW]
-    uint32_t *pix_last;      // [sum HW] list position after the last blend
+    uint32_t *pix_last;      // [sum HW] list position where the pixel stopped (else the list's length)
     uint32_t *pix_neval;     // [2][sum HW] stats pass: in-footprint entries up to the stop, and blended ones
     // backward
     double *g2m;             // [M*3] moments m_xx, m_xy, m_yy of dL/dpower over the pixels' offsets from

@@ -557,8 +557,7 @@ __device__ __forceinline__ uint32_t sort_excl_scan(uint32_t v, uint32_t *smem) {
 // behind its write-out; four barriers per tile.  The ALU pipe is the busiest
 // (the ballots; half of its slots), so whole tiles skip the tests of the end
 // and a key's place takes one shared load (8M 32-bit pairs, four passes: 311
-// -> 297 us; a step of twelve views, 40M
-// pairs: 6,242 -> 6,206 us).
+// -> 297 us; a step of twelve views, 40M pairs: 6,242 -> 6,206 us).
 template <int ITEMS, int NB, bool kLateVals>
 __device__ __forceinline__ void radix_downsweep(const uint32_t *__restrict__ keys_in,
                                                 const uint32_t *__restrict__ vals_in, uint32_t *__restrict__ keys_out,
