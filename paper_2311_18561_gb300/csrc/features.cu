@@ -23,7 +23,8 @@ int feat_count(int mask, int n_sem) {
 // their sums fit the registers (24 channels); two below, where the longest
 // walk bounds the pass (23 channels, four / two: 1920x1280 with 1.5M
 // Gaussians 708 / 1033 us, 1242x800 with 100k 169 / 209, 1242x375 with 300k
-// 577 / 400, 640x480 with 200k 408 / 227).
+// 577 / 400, 640x480 with 200k 408 / 227; packed by channels since: 654, 158,
+// 368 and 210).
 constexpr int kFeatWide = 40, kFeatWideGroups = 6;
 
 void launch_composite_feat(const Params &p, cudaStream_t s) {

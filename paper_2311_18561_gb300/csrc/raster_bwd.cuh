@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
     __shared__ RawRecords raw;
     __shared__ Staged Sg;
     __shared__ TermBuffer<NT> buf;
-    __shared__ StagedFeats<NG, false> F;
+    __shared__ StagedFeats<NG> F;
     __shared__ FeatBuffer<NG, (NG > 0 ? kBwdUnrollFeat : 1)> fbuf;
     const int lane = threadIdx.x;
     const BlockGeom G = block_geom<PX>(P);
@@ -284,10 +284,9 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
             odd |= !(fabsf(e.gC0) + fabsf(e.gC1) + fabsf(e.gC2) + fabsf(e.gD) + fabsf(e.gO) + fabsf(e.S) < 1e15f);
     }
     sky.flush(V);
-    // output gradients of the extra channels (negated), pairs of channels: the
-    // arithmetic on them is packed by channels, which needs no value twice and
-    // adds no pixels' halves up per channel (1242x1242 with 300k Gaussians, 23
-    // channels: 1025 us packed by pixels, 838 us by channels)
+    // output gradients of the extra channels (negated), pairs of channels: packed
+    // by pixels instead, every channel's two halves have to be added up
+    // (1242x1242 with 300k Gaussians, 23 channels: 1025 us, by channels 838)
     float2 nF[PX][NG > 0 ? 2 * NG : 1];
     if constexpr (NG > 0) {
         const size_t HW = (size_t)V.W * V.H;

@@ -24,9 +24,10 @@ constexpr int kFwdWide = 64;
 // With one pixel per lane (four entries together: 156 us on those views,
 // eight 164 us).
 constexpr int kFwdWarps1 = 24, kFwdUnroll1 = 4;
-// With extra channels: two pixels per lane (their sums fill the registers).
-// The longest walk bounds the pass here too (23 channels, 1242x375, 200k
-// Gaussians: 330 us with two entries together, 282 us with four).
+// With extra channels (two or four pixels per lane; their sums, packed by
+// pairs of channels, fill the registers).  The longest walk bounds the pass
+// here too (23 channels, 1242x375, 200k Gaussians: 330 us with two entries
+// together, 282 us with four).
 constexpr int kFwdWarpsFeat = 8, kFwdUnrollFeat = 4;
 
 // Writes the images (and the saved per-pixel state) of a thread's PX pixels.
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kFwdWarpsFeat : PX == 4 ? kFwdWar
     constexpr uint32_t ALL = (1u << PX) - 1u;
     __shared__ RawRecords raw;
     __shared__ Staged S;
-    __shared__ StagedFeats<NG, true> F;
+    __shared__ StagedFeats<NG> F;
     const int lane = threadIdx.x;
     const BlockGeom G = block_geom<PX>(P);
     const ViewDesc &V = *G.V;
@@ -103,12 +104,12 @@ __global__ void __launch_bounds__(32, NG > 0 ? kFwdWarpsFeat : PX == 4 ? kFwdWar
         T[q] = make_float2(1.0f, 1.0f);
         C0[q] = C1[q] = C2[q] = D[q] = O[q] = nzero2;
     }
-    float2 fa[NP][NG > 0 ? 4 * NG : 1];  // extra channels' sums (negated)
+    float2 fa[PX][NG > 0 ? 2 * NG : 1];  // extra channels' sums (negated), pairs of channels
     if constexpr (NG > 0) {
 #pragma unroll
-        for (int q = 0; q < NP; q++)
+        for (int p = 0; p < PX; p++)
 #pragma unroll
-            for (int c = 0; c < 4 * NG; c++) fa[q][c] = nzero2;
+            for (int c = 0; c < 2 * NG; c++) fa[p][c] = nzero2;
     }
     const uint32_t len = r.y - r.x;
 #pragma unroll
@@ -200,8 +201,8 @@ __global__ void __launch_bounds__(32, NG > 0 ? kFwdWarpsFeat : PX == 4 ? kFwdWar
                             if constexpr (NG > 0) {
 #pragma unroll
                                 for (int c = 0; c < 4 * NG; c++) {
-                                    float &a = p & 1 ? fa[p / 2][c].y : fa[p / 2][c].x;
-                                    a = __fmaf_rn(F.f[k + u][c].x, nw, a);
+                                    float &a = c & 1 ? fa[p][c / 2].y : fa[p][c / 2].x;
+                                    a = __fmaf_rn(F.f[k + u][c], nw, a);
                                 }
                             }
                         };
@@ -274,12 +275,13 @@ __global__ void __launch_bounds__(32, NG > 0 ? kFwdWarpsFeat : PX == 4 ? kFwdWar
                 }
                 if constexpr (NG > 0) {
 #pragma unroll
-                    for (int c = 0; c < 4 * NG; c += 2) {
-                        const float4 f = reinterpret_cast<const float4 *>(&F.f[k + u][c])[0];
+                    for (int g = 0; g < NG; g++) {  // (packed by pixels, every value staged twice: 8 % more)
+                        const float4 f = reinterpret_cast<const float4 *>(&F.f[k + u][0])[g];
 #pragma unroll
-                        for (int q = 0; q < NP; q++) {
-                            fa[q][c] = fma2(make_float2(f.x, f.y), nw[u][q], fa[q][c]);
-                            fa[q][c + 1] = fma2(make_float2(f.z, f.w), nw[u][q], fa[q][c + 1]);
+                        for (int p = 0; p < PX; p++) {
+                            const float w = p & 1 ? nw[u][p / 2].y : nw[u][p / 2].x;
+                            fa[p][2 * g] = fma2(make_float2(f.x, f.y), make_float2(w, w), fa[p][2 * g]);
+                            fa[p][2 * g + 1] = fma2(make_float2(f.z, f.w), make_float2(w, w), fa[p][2 * g + 1]);
                         }
                     }
                 }
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kFwdWarpsFeat : PX == 4 ? kFwdWar
             float *out = V.out_feat + (size_t)(G.py0 + p) * V.W + G.px;
 #pragma unroll
             for (int c = 0; c < 4 * NG; c++)
-                if (c < P.n_feat) out[c * HW] = -(p & 1 ? fa[p / 2][c].y : fa[p / 2][c].x);
+                if (c < P.n_feat) out[c * HW] = -(c & 1 ? fa[p][c / 2].y : fa[p][c / 2].x);
         }
     }
     if (P.tile_walk) {  // how far the tile's adjoint walks, for its launch order
