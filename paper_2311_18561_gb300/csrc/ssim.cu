@@ -27,6 +27,8 @@
 // the scalar filter did.
 #include <cooperative_groups.h>
 
+#include <utility>
+
 #include "pvg_internal.cuh"
 
 namespace pvg {
@@ -315,11 +317,15 @@ __global__ void __launch_bounds__(kThreads, 3) k_rgb_loss(const float *__restric
 
 // loss[0..2] = (L, L1, SSIM) from the per-CTA partial sums, added in a
 // fixed order in double precision by one cluster of kFinish CTAs (the 64-bit
-// adders are few: one CTA takes 13 us for 7,200 partial sums).
+// adders are few: one CTA takes 13 us for 7,200 partial sums).  Another CTA's
+// shared memory may be written only once that CTA has started: every CTA
+// arrives at a cluster barrier on entry and waits for it before its store.
 constexpr int kFinish = 8, kFinishThreads = 256;
 
 __global__ void __cluster_dims__(kFinish, 1, 1) __launch_bounds__(kFinishThreads)
     k_rgb_loss_finish(const float2 *__restrict__ partial, int n, double inv_n, float lambda_r, float *loss) {
+    auto cluster = cooperative_groups::this_cluster();
+    auto started = cluster.barrier_arrive();
     pdl_enter();
     __shared__ double s_warp[2][kFinishThreads / 32];
     __shared__ double s_cta[2][kFinish];  // CTA 0's: every CTA's sums
@@ -338,7 +344,7 @@ __global__ void __cluster_dims__(kFinish, 1, 1) __launch_bounds__(kFinishThreads
         s_warp[1][threadIdx.x >> 5] = b;
     }
     __syncthreads();
-    auto cluster = cooperative_groups::this_cluster();
+    cluster.barrier_wait(std::move(started));
     if (threadIdx.x < 2) {
         double t = 0.0;
         for (int w = 0; w < kFinishThreads / 32; w++) t += s_warp[threadIdx.x][w];
