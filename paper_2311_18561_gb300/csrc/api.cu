@@ -15,7 +15,6 @@
 // (a frame of at most kSmallFrameItems items takes one CTA per sorting stage)
 // Backward: k_composite_bwd (image-space gradients per record) and
 // k_preprocess_bwd (parameter gradients).
-#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -219,7 +218,7 @@ struct pvg_ctx {
     DevBuf alt_keys, alt_vals;   // [NV] depth sort ping-pong
     DevBuf pair_keys, pair_keys2, pair_vals2;  // [K]
     DevBuf vis_off;              // [NV]
-    DevBuf chunk_start;          // [K / 2048 + 1]
+    DevBuf chunk_start;          // first item of each pair chunk (emit_chunks)
     DevBuf temp;
     DevBuf sort_n;               // u32: element count of pvg_sort_pairs
     DevBuf loss_partials;        // float2 per CTA of pvg_rgb_loss
@@ -576,15 +575,14 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
     PVG_TRY(ensure_c(f->pix_last, sizeof(uint32_t) * pix, capturing));
     PVG_TRY(ensure_c(f->pix_neval, sizeof(uint32_t) * 2 * (size_t)pix, capturing));
     const bool small = NV <= kSmallFrameItems && tiles <= kSmallFrameTiles;  // one CTA per sorting stage
-    if (small)
-        PVG_TRY(ensure_c(x->chunk_start,
-                         sizeof(uint32_t) * small_emit_chunks(NV, tiles, x->cfg.sync_sizes ? 0xffffffffu
-                                                                                           : (uint32_t)x->cfg.pair_capacity),
-                         capturing));
     uint32_t pair_cap;
     if (x->cfg.sync_sizes) {
         pair_cap = (uint32_t)(f->pair_vals.bytes / sizeof(uint32_t));
+        // (a small frame's pairs are counted and their chunks marked in one launch)
+        if (small) PVG_TRY(ensure_c(x->chunk_start, sizeof(uint32_t) * emit_chunks(NV * tiles), capturing));
     } else {
+        // sized by the capacity alone: a captured graph holds these buffers, so
+        // no later frame on the context may move them
         pair_cap = (uint32_t)x->cfg.pair_capacity;
         PVG_TRY(ensure_c(f->pair_vals, sizeof(uint32_t) * (size_t)pair_cap, capturing));
         PVG_TRY(ensure_c(x->pair_keys, sizeof(uint32_t) * (size_t)pair_cap, capturing));
@@ -824,9 +822,7 @@ pvg_status_t serve_reserve(pvg_ctx_t *x, pvg_frame_t *f, uint64_t items, uint64_
     PVG_TRY(ensure(f->pix_neval, sizeof(uint32_t) * 2 * pix));
     for (DevBuf *b : {&f->pair_vals, &x->pair_keys, &x->pair_keys2, &x->pair_vals2})
         PVG_TRY(ensure(*b, sizeof(uint32_t) * pairs));
-    PVG_TRY(ensure(x->chunk_start, sizeof(uint32_t) * std::max(emit_chunks((uint32_t)pairs),
-                                                               small_emit_chunks(kSmallFrameItems, kSmallFrameTiles,
-                                                                                 (uint32_t)pairs))));
+    PVG_TRY(ensure(x->chunk_start, sizeof(uint32_t) * emit_chunks((uint32_t)pairs)));
     PVG_TRY(ensure(f->stage_fwd->dev, sizeof(ViewDesc) * (size_t)max_views));
     return PVG_OK;
 }

@@ -110,7 +110,7 @@ struct Params {
     uint32_t *vis_tile;      // [M] several views: id of the rectangle's first tile (in item_zkey's space,
                              // dead after the compaction)
     uint32_t *vis_stride;    // [M] several views: tiles per row of the view (in item_cnt's space)
-    uint32_t *chunk_start;   // [K / 2048 + 1] first item of each pair chunk
+    uint32_t *chunk_start;   // [emit_chunks(capacity)] first item of each pair chunk
     // pairs
     uint32_t *pair_keys;     // [K] tile ids (sorted in place via ping-pong)
     uint32_t *pair_vals;     // [K]
@@ -488,13 +488,14 @@ void radix_sort_pairs(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32
                       cudaStream_t s, bool *result_in_alt, uint32_t *inv_out = nullptr, bool first_hist = false);
 void scan_count_pairs(const Params &p, void *temp, cudaStream_t s);
 void scan_emit_pairs(const Params &p, void *temp, cudaStream_t s);
+// entries of chunk_start for a capacity of pairs, whatever the frame's size
 size_t emit_chunks(uint32_t capacity);
 // Small frames: the same stages, one CTA each.  At most kSmallFrameItems
 // items; the tile sort also at most as many pairs of capacity.
 constexpr uint32_t kSmallFrameItems = 8192, kSmallFrameTiles = 65536;
+static_assert((uint64_t)kSmallFrameItems * kSmallFrameTiles < 1ull << 32, "their pairs fit 32 bits");
 constexpr uint32_t kSmallOrderTiles = 8192;  // above it the launch order is the cluster's
 cudaError_t set_small_frame_smem();
-size_t small_emit_chunks(uint64_t n_items, uint64_t tiles, uint32_t capacity);
 void small_depth_sort(const Params &p, cudaStream_t s);
 void small_count_pairs(const Params &p, cudaStream_t s);
 // count_digits: the general tile sort follows (its first digit histogram)

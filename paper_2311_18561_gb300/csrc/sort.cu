@@ -863,7 +863,9 @@ void scan_count_pairs(const Params &p, void *temp, cudaStream_t s) {
     pdl_launch(k_scan_partials, 1, 1024, 0, s, t.partials, G, &p.counters[1], p.pair_capacity, &p.counters[2]);
 }
 
-size_t emit_chunks(uint32_t capacity) { return (capacity + kEmitChunk - 1) / kEmitChunk + 1; }
+// the small frames' chunks are the shorter ones
+static_assert(kEmitChunkSmall <= kEmitChunk, "entries for either chunk length");
+size_t emit_chunks(uint32_t capacity) { return capacity / kEmitChunkSmall + 2; }
 
 void scan_emit_pairs(const Params &p, void *temp, cudaStream_t s) {
     TempLayout t = temp_layout(temp);
@@ -1190,10 +1192,6 @@ cudaError_t set_small_frame_smem() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_small_tile_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OneSmem));
     return e;
-}
-
-size_t small_emit_chunks(uint64_t n_items, uint64_t tiles, uint32_t capacity) {
-    return (size_t)(std::min<uint64_t>(n_items * tiles, capacity) / kEmitChunkSmall + 2);
 }
 
 void small_depth_sort(const Params &p, cudaStream_t s) {
