@@ -264,7 +264,10 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
     uint32_t last[PX];
     uint32_t walk = 0;
     SkyScatter sky;
-    bool odd = false;  // non-finite or huge output gradients: pixels one at a time
+    // pixels one at a time: non-finite or huge output gradients, and from the
+    // first 32 entries on that hold such a term, behind which a pixel's suffix
+    // sum may be infinite (carried by entry it costs the adjoint 1 %)
+    bool odd = false;
 #pragma unroll
     for (int q = 0; q < NP; q++) {
         fy[q] = make_float2((float)(G.py0 + 2 * q) + 0.5f, (float)(G.py0 + 2 * q + 1) + 0.5f);
@@ -281,7 +284,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
         last[2 * q + 1] = b.last;
         walk = max(walk, max(a.last, b.last));
         for (const PixelAdjoint &e : {a, b})
-            odd |= !(fabsf(e.gC0) + fabsf(e.gC1) + fabsf(e.gC2) + fabsf(e.gD) + fabsf(e.gO) + fabsf(e.S) < 1e15f);
+            odd |= !(fabsf(e.gC0) + fabsf(e.gC1) + fabsf(e.gC2) + fabsf(e.gD) + fabsf(e.gO) + fabsf(e.S) < kGradBound);
     }
     sky.flush(V);
     // output gradients of the extra channels (negated), pairs of channels: packed
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
             for (int c = 0; c < 2 * NG; c++) {
                 nF[p][c].x = in && 2 * c < P.n_feat ? -src[2 * c * HW] : 0.f;
                 nF[p][c].y = in && 2 * c + 1 < P.n_feat ? -src[(2 * c + 1) * HW] : 0.f;
-                odd |= !(fabsf(nF[p][c].x) + fabsf(nF[p][c].y) < 1e15f);
+                odd |= !(fabsf(nF[p][c].x) + fabsf(nF[p][c].y) < kGradBound);
             }
         }
     }
@@ -326,6 +329,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
             if (m0 != kNoRecord) i0 = P.sgid[m0] - V.item_base;
             stage_feats<NG, kSlots>(P, V, Sg, F, hits, lane);
         }
+        odd |= __any_sync(0xffffffffu, lane < hits && (__float_as_uint(Sg.a[lane].w) & kOddEntry));
         for (int base = (hits - 1) & ~(kSlots - 1); base >= 0; base -= kSlots) {
             uint32_t valid = 0;  // slots that hold an entry's terms
 #pragma unroll 1
@@ -370,7 +374,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
                     if constexpr (kAux) z2 = Sg.e[k];
                     float A0, M1, M2, c0, c1, c2, zs = 0.f;
                     float2 nwf[NP];  // the pixels' weights (negated)
-                    if (!odd && !(pf[u] & kOddEntry)) {
+                    if (!odd) {
                         float2 A0v, M1v, M2v, c0v, c1v, c2v, zv;
                         auto pairs = [&](auto capped) {
                             constexpr bool kCap = decltype(capped)::value;
@@ -470,7 +474,7 @@ __global__ void __launch_bounds__(32, NG > 0 ? kBwdWarpsFeat : BwdTune<PX>::kWar
                     }
                     if constexpr (NG > 0) {
                         float2 gf[2 * NG];
-                        if (!odd && !(pf[u] & kOddEntry)) {
+                        if (!odd) {
 #pragma unroll
                             for (int p = 0; p < PX; p++) {
                                 const float w = p & 1 ? nwf[p / 2].y : nwf[p / 2].x;

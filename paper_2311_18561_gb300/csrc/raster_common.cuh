@@ -70,9 +70,17 @@ __device__ __forceinline__ bool block_hit(float u, float v, float ap, float bp, 
 }
 
 // flags beside an entry's list position
-constexpr uint32_t kOddEntry = 0x80000000u;     // non-finite terms: pixels one at a time
+constexpr uint32_t kOddEntry = 0x80000000u;     // non-finite or huge terms: pixels one at a time
 constexpr uint32_t kCappedEntry = 0x40000000u;  // o~ may exceed the alpha cap
 constexpr uint32_t kPosMask = 0x3fffffffu;      // a list of 2^30 entries does not fit the device memory
+
+// Below these bounds of an entry's terms and channel values and of a pixel's
+// output gradients, the arithmetic that gives a pixel without a blend the
+// weight zero meets finite values only: X, a sum of at most 41 products of one
+// with the other, and the adjoint's suffix sum, a weighted mean of such X.
+// Whatever lies above takes pixels one at a time.
+constexpr float kTermBound = 1e18f, kGradBound = 1e15f;
+static_assert(41.0 * kTermBound * kGradBound < 1e36, "two orders below the largest float");
 
 constexpr int kStagedPlaces = 32;
 
@@ -157,10 +165,9 @@ __device__ __forceinline__ int stage_hits(const RawRecords &raw, Stage &S, bool 
     const uint32_t mask = __ballot_sync(0xffffffffu, hit);
     if (hit) {
         const int k = __popc(mask & ((1u << lane) - 1u));
-        // finite: no term is NaN or infinite, so that 0 weights keep sums unchanged
         const float s = fabsf(a.x) + fabsf(a.y) + fabsf(a.z) + fabsf(a.w) + fabsf(b.x) + fabsf(b.y) + fabsf(c.x) +
                         fabsf(c.y) + fabsf(c.z) + fabsf(c.w);
-        pos |= (s < 1e30f ? 0u : kOddEntry) | (b.y <= kUncappedOpacity ? 0u : kCappedEntry);
+        pos |= (s < kTermBound ? 0u : kOddEntry) | (b.y <= kUncappedOpacity ? 0u : kCappedEntry);
         S.put(k, a, b, c, pos, m);
         if (items) items[k] = item;
     }
@@ -227,7 +234,7 @@ __device__ __forceinline__ void stage_feats(const Params &P, const ViewDesc &V, 
             put(vel.z * w);
         }
         if (P.feat_mask & kFeatRho) put(fminf(rho, 2.0f));
-        if (!(bad < 1e30f)) S.a[lane].w = __uint_as_float(__float_as_uint(S.a[lane].w) | kOddEntry);
+        if (!(bad < kTermBound)) S.a[lane].w = __uint_as_float(__float_as_uint(S.a[lane].w) | kOddEntry);
     }
     for (int k = hits; k < places; k++)
         for (int c = lane; c < 4 * NG; c += 32) F.f[k][c] = 0.f;
@@ -237,7 +244,7 @@ __device__ __forceinline__ void stage_feats(const Params &P, const ViewDesc &V, 
         if (lane < n_sem)
 #pragma unroll 4
             for (int k = 0; k < hits; k++) {
-                bad |= fabsf(F.f[k][c0 + lane]) < 1e30f ? 0u : 1u << k;
+                bad |= fabsf(F.f[k][c0 + lane]) < kTermBound ? 0u : 1u << k;
             }
         bad = __reduce_or_sync(0xffffffffu, bad);
         if ((bad >> lane) & 1u) S.a[lane].w = __uint_as_float(__float_as_uint(S.a[lane].w) | kOddEntry);
