@@ -322,6 +322,9 @@ class PVGRender(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, g_rgb, g_depth, g_alpha):
+        if torch.cuda.is_current_stream_capturing():
+            # the graph would go on using a frame that other renders are lent
+            raise abi.PVGError(abi.PVG_ERR_INVALID, "pvg_render_bwd")
         saved = ctx.saved_tensors
         scene_t = dict(zip(PARAM_NAMES, saved))
         if ctx.has_sky:

@@ -1,0 +1,62 @@
+"""The idle frames that a renderer keeps for render_differentiable are never
+left to a captured backward pass.
+"""
+import pytest
+import torch
+
+from paper_2311_18561_gb300 import abi
+from paper_2311_18561_gb300 import render as R
+from paper_2311_18561_gb300 import synth
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+CAM = synth.plain_camera(64, 48, t=0.3)
+
+
+@pytest.fixture(autouse=True)
+def _clear_hook():
+    yield
+    abi.lib().pvg_debug_fail_allocations(0)
+
+
+@pytest.fixture(scope="module")
+def scene():
+    return R.scene_to_device(synth.make_plain_scene(seed=2, n=500))
+
+
+def _forward(st, r, cam=CAM):
+    p = {k: v.clone().requires_grad_(True) for k, v in st.items()}
+    return p, R.render_differentiable(p, cam, r)
+
+
+def _backward(p, out, **kw):
+    return torch.autograd.grad(out, list(p.values()), [torch.ones_like(o) for o in out], **kw)
+
+
+def _step(st, r):
+    g = _backward(*_forward(st, r))
+    torch.cuda.synchronize()
+    return g
+
+
+def test_a_captured_backward_pass_is_refused(scene):
+    """A graph would keep using a frame that other renders are lent."""
+    r = R.Renderer(sync_sizes=False, pair_capacity=1 << 20)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        want = _step(scene, r)
+        p, out = _forward(scene, r)
+        seeds = [torch.ones_like(o) for o in out]
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with pytest.raises(abi.PVGError) as e:
+        with torch.cuda.graph(graph, stream=stream):
+            torch.autograd.grad(out, list(p.values()), seeds, retain_graph=True)
+    assert e.value.status == 1 and not r._frames
+    with torch.cuda.stream(stream):  # the render can still be differentiated
+        got = torch.autograd.grad(out, list(p.values()), seeds)
+    torch.cuda.synchronize()
+    for a, b in zip(want, got):
+        assert torch.linalg.norm(a - b) <= 1e-5 * torch.linalg.norm(a)
+    r.close()
