@@ -467,6 +467,10 @@ uint64_t pvg_kernel_launches(void);
  * grids with them (cudaDevAttrMultiProcessorCount, read once per device). */
 int32_t pvg_device_sm_count(void);
 
+/* *id = a number of the stream that no other stream of the process ever has
+ * (a handle is used again once its stream is destroyed). */
+pvg_status_t pvg_stream_id(void *stream, uint64_t *id);
+
 /* FP32 throughput probe, the measured peak of the compositing kernels'
  * roofline (not part of the rendering path): `blocks` blocks of 256
  * threads, every thread running `iters` rounds of 128 fused multiply-adds

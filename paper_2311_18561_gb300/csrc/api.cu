@@ -1058,6 +1058,14 @@ extern "C" pvg_status_t pvg_frame_export(pvg_frame_t *f, uint32_t *sorted_gid, u
 
 extern "C" uint64_t pvg_kernel_launches(void) { return pvg::g_launches.load(); }
 
+extern "C" pvg_status_t pvg_stream_id(void *stream, uint64_t *id) {
+    if (!id) return PVG_ERR_INVALID;
+    unsigned long long v = 0;
+    PVG_CUDA(cudaStreamGetId((cudaStream_t)stream, &v));
+    *id = v;
+    return PVG_OK;
+}
+
 extern "C" pvg_status_t pvg_profile_enable(pvg_ctx_t *x, int on) {
     if (!x) return PVG_ERR_INVALID;
     x->timer.on = on != 0;

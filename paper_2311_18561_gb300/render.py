@@ -96,6 +96,19 @@ def _stream_ptr(stream=None):
     return C.c_void_p(st.cuda_stream)
 
 
+def _stream_key(stream):
+    """Equal for two uses of a stream, different for two streams: torch never
+    destroys its own streams, whose handles tell them apart; a caller's
+    (``ExternalStream``: torch's id of it is the handle) may be destroyed and
+    its handle given to another."""
+    handle = stream.cuda_stream
+    if not handle or stream.stream_id != handle:
+        return handle, 0
+    i = C.c_uint64()
+    abi.check(abi.lib().pvg_stream_id(handle, C.byref(i)), "pvg_stream_id")
+    return handle, i.value
+
+
 class Renderer:
     """Owns one ``pvg_ctx_t`` (workspace) on the current CUDA device."""
 
@@ -255,7 +268,8 @@ class _FrameLease:
     frames or new, and given back by ``release`` (or when dropped).  A frame
     holds some 20 device buffers, and creating and freeing them was most of a
     small differentiable render.  An idle frame is only lent to the stream
-    that used it last, behind whose work it is free.  A renderer keeps at
+    that used it last, behind whose work it is free: the stream itself, and
+    not one that was given a destroyed stream's handle.  A renderer keeps at
     most ``KEEP`` idle frames and frees them with itself; a lease taken while
     the stream is being captured is a frame of its own."""
 
@@ -264,15 +278,16 @@ class _FrameLease:
     def __init__(self, renderer):
         self.renderer = renderer
         self.frame = None
-        self.stream = torch.cuda.current_stream().cuda_stream
+        self.stream = torch.cuda.current_stream()
         self.own = torch.cuda.is_current_stream_capturing()
         if not self.own:
+            self.key = _stream_key(self.stream)
             for _ in range(len(renderer._frames)):
                 try:
                     stream, frame = renderer._frames.pop()
                 except IndexError:  # another thread's
                     break
-                if stream == self.stream:
+                if frame.stream_key == self.key:
                     self.frame = frame
                     break
                 renderer._frames.insert(0, (stream, frame))
@@ -284,15 +299,18 @@ class _FrameLease:
         return self.frame.handle if self.frame is not None else None
 
     def release(self, stream=None):
-        """``stream``: the last call's, if it was not the lease's."""
+        """``stream``: the last call's, if it may not be the lease's."""
         frame, self.frame = self.frame, None
         if frame is None:
             return
         r = self.renderer
-        if self.own or r.handle is None or stream not in (None, self.stream) or len(r._frames) >= self.KEEP:
+        handle = self.stream.cuda_stream
+        if (self.own or r.handle is None or (stream is not None and stream.cuda_stream != handle)
+                or len(r._frames) >= self.KEEP):
             frame.close()
         else:
-            r._frames.append((self.stream, frame))
+            frame.stream_key = self.key
+            r._frames.append((handle, frame))
 
     def __del__(self):
         try:
@@ -314,7 +332,7 @@ class PVGRender(torch.autograd.Function):
         if sky is not None:
             scene_t["sky"] = sky.contiguous()
         frame = _FrameLease(renderer)
-        out = renderer.forward(scene_t, [cam], frame=frame)[0]
+        out = renderer.forward(scene_t, [cam], frame=frame, stream=frame.stream)[0]
         ctx.cam, ctx.renderer, ctx.frame = cam, renderer, frame
         ctx.has_sky = sky is not None
         ctx.save_for_backward(*[scene_t[k] for k in PARAM_NAMES], *([scene_t["sky"]] if sky is not None else []))
@@ -329,9 +347,10 @@ class PVGRender(torch.autograd.Function):
         scene_t = dict(zip(PARAM_NAMES, saved))
         if ctx.has_sky:
             scene_t["sky"] = saved[len(PARAM_NAMES)]
+        stream = torch.cuda.current_stream()
         grads = ctx.renderer.backward(scene_t, [ctx.cam], ctx.frame,
-                                      [dict(rgb=g_rgb, depth=g_depth, alpha=g_alpha)])
-        ctx.frame.release(torch.cuda.current_stream().cuda_stream)
+                                      [dict(rgb=g_rgb, depth=g_depth, alpha=g_alpha)], stream=stream)
+        ctx.frame.release(stream)
         return (None, None) + tuple(grads[k] for k in PARAM_NAMES) + (grads.get("sky"),)
 
 

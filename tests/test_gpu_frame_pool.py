@@ -1,6 +1,9 @@
 """The idle frames that a renderer keeps for render_differentiable are never
-left to a captured backward pass.
+lent to a stream that only has the handle of a destroyed one, and never left
+to a captured backward pass.
 """
+import ctypes
+
 import pytest
 import torch
 
@@ -37,6 +40,42 @@ def _step(st, r):
     g = _backward(*_forward(st, r))
     torch.cuda.synchronize()
     return g
+
+
+def _external_stream():
+    """(handle, destroy): a stream of the caller's own."""
+    rt = torch.cuda.cudart()
+    s = ctypes.c_void_p()
+    assert int(rt.cudaStreamCreate(ctypes.addressof(s))) == 0
+    return s.value, lambda: rt.cudaStreamDestroy(s.value)
+
+
+def test_a_destroyed_streams_handle_does_not_lend_its_frames(scene):
+    r = R.Renderer()
+    handle, destroy = _external_stream()
+    with torch.cuda.stream(torch.cuda.ExternalStream(handle)):
+        _step(scene, r)
+        (idle,) = [f for _, f in r._frames]
+        lease = R._FrameLease(r)
+        assert lease.frame is idle  # the same stream
+        lease.release()
+    torch.cuda.synchronize()
+    destroy()
+    made = []
+    for _ in range(64):
+        made.append(_external_stream())
+        if made[-1][0] == handle:
+            break
+    try:
+        if made[-1][0] != handle:
+            pytest.skip("no new stream got the destroyed one's handle")
+        with torch.cuda.stream(torch.cuda.ExternalStream(handle)):
+            assert R._FrameLease(r).frame is not idle
+    finally:
+        torch.cuda.synchronize()
+        r.close()
+        for _, d in made:
+            d()
 
 
 def test_a_captured_backward_pass_is_refused(scene):
