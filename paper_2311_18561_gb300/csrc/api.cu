@@ -292,7 +292,13 @@ extern "C" pvg_status_t pvg_frame_create(pvg_frame_t **frame) {
 
 extern "C" void pvg_frame_destroy(pvg_frame_t *f) {
     if (!f) return;
-    if (f->stream) cudaStreamSynchronize(f->stream);
+    // the stream of its last call may be gone, so its handle is not used: the
+    // frame's device is waited for, as the frees below do in any case
+    int device = f->device;
+    cudaGetDevice(&device);
+    if (device != f->device) cudaSetDevice(f->device);
+    cudaDeviceSynchronize();
+    if (device != f->device) cudaSetDevice(device);
     for (DevBuf *b : {&f->counters, &f->sgid, &f->inv, &f->szkey, &f->rec, &f->ell, &f->rowtab, &f->rect, &f->vis_cnt, &f->pair_vals,
                       &f->ranges, &f->tile_order, &f->tile_walk, &f->tile_order_bwd, &f->pix_T, &f->pix_last, &f->pix_neval, &f->g2d, &f->gfeat})
         release(*b);

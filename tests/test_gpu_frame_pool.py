@@ -1,6 +1,6 @@
 """The idle frames that a renderer keeps for render_differentiable are never
-lent to a stream that only has the handle of a destroyed one, and never left
-to a captured backward pass.
+lent to a stream that only has the handle of a destroyed one, outlive the
+stream that used them, and are never left to a captured backward pass.
 """
 import ctypes
 
@@ -51,6 +51,8 @@ def _external_stream():
 
 
 def test_a_destroyed_streams_handle_does_not_lend_its_frames(scene):
+    """Whether a new stream gets a destroyed one's handle is the driver's
+    choice, so the idle frame is entered under a new stream's handle."""
     r = R.Renderer()
     handle, destroy = _external_stream()
     with torch.cuda.stream(torch.cuda.ExternalStream(handle)):
@@ -61,21 +63,34 @@ def test_a_destroyed_streams_handle_does_not_lend_its_frames(scene):
         lease.release()
     torch.cuda.synchronize()
     destroy()
-    made = []
-    for _ in range(64):
-        made.append(_external_stream())
-        if made[-1][0] == handle:
-            break
+    made = [_external_stream() for _ in range(8)]
     try:
-        if made[-1][0] != handle:
-            pytest.skip("no new stream got the destroyed one's handle")
-        with torch.cuda.stream(torch.cuda.ExternalStream(handle)):
+        ids = {idle.stream_key[1]} | {R._stream_key(torch.cuda.ExternalStream(h))[1] for h, _ in made}
+        assert 0 not in ids and len(ids) == len(made) + 1
+        new = made[0][0]
+        with torch.cuda.stream(torch.cuda.ExternalStream(new)):
+            r._frames[:] = [(new, idle)]
+            idle.stream_key = (new, idle.stream_key[1])
             assert R._FrameLease(r).frame is not idle
     finally:
         torch.cuda.synchronize()
         r.close()
         for _, d in made:
             d()
+
+
+def test_frames_outlive_the_stream_that_used_them(scene):
+    cam2 = synth.plain_camera(48, 32)
+    r, fr = R.Renderer(), R.Frame()
+    handle, destroy = _external_stream()
+    with torch.cuda.stream(torch.cuda.ExternalStream(handle)):
+        _step(scene, r)
+        r.forward(scene, [cam2], frame=fr)
+    torch.cuda.synchronize()
+    assert len(r._frames) == 1
+    destroy()
+    fr.close()
+    r.close()
 
 
 def test_a_captured_backward_pass_is_refused(scene):
