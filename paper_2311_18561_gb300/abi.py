@@ -13,7 +13,7 @@ from . import build as _build
 
 _LIB = None
 
-PVG_OK, PVG_ERR_INVALID = 0, 1
+PVG_OK, PVG_ERR_INVALID, PVG_ERR_OOM = 0, 1, 2
 STATUS = {0: "PVG_OK", 1: "PVG_ERR_INVALID", 2: "PVG_ERR_OOM", 3: "PVG_ERR_BUSY", 4: "PVG_ERR_TIMEOUT",
           5: "PVG_ERR_CUDA", 6: "PVG_ERR_OVERFLOW", 7: "PVG_ERR_NOT_FOUND"}
 

@@ -120,14 +120,32 @@ class Renderer:
         abi.check(self._lib.pvg_create(C.byref(h), C.byref(self.cfg)), "pvg_create")
         self.handle = h
         self.device = torch.cuda.current_device()
-        self._frames = []  # (stream, frame): idle frames of render_differentiable
+        self._frames = []  # (stream, frame): idle frames of render_differentiable, the last used last
 
     def close(self):
         if self.handle:
-            while self._frames:
-                self._frames.pop()[1].close()
+            self.free_idle_frames()
             self._lib.pvg_destroy(self.handle)
             self.handle = None
+
+    def free_idle_frames(self):
+        """Frees the frames kept for :func:`render_differentiable` (as large
+        as their largest renders); the next such render makes one again."""
+        while self._frames:
+            try:
+                self._frames.pop()[1].close()
+            except IndexError:  # another thread's
+                break
+
+    def _run(self, name, *args):
+        """A library call with this renderer's workspace; out of device
+        memory, once more without the idle frames."""
+        fn = getattr(self._lib, name)
+        st = fn(self.handle, *args)
+        if st == abi.PVG_ERR_OOM and self._frames:
+            self.free_idle_frames()
+            st = fn(self.handle, *args)
+        abi.check(st, name)
 
     def __del__(self):
         try:
@@ -165,9 +183,8 @@ class Renderer:
         ca = abi.cameras(cams)
         imgs = (abi.Image * len(cams))()
         _fill_images(imgs, outs, features)
-        st = self._lib.pvg_render_fwd(self.handle, C.byref(sc), ca, len(cams), imgs,
-                                      frame.handle if frame is not None else None, _stream_ptr(stream))
-        abi.check(st, "pvg_render_fwd")
+        self._run("pvg_render_fwd", C.byref(sc), ca, len(cams), imgs,
+                  frame.handle if frame is not None else None, _stream_ptr(stream))
         return outs
 
     def backward(self, scene_t, cams, frame, grads_out, stream=None, grads=None):
@@ -192,9 +209,7 @@ class Renderer:
             for name in ("rgb", "depth", "alpha", "feat"):
                 t = d.get(name)
                 setattr(dl[k], name, t.contiguous().data_ptr() if t is not None else None)
-        st = self._lib.pvg_render_bwd(self.handle, C.byref(sc), ca, len(cams), frame.handle, dl, C.byref(g),
-                                      _stream_ptr(stream))
-        abi.check(st, "pvg_render_bwd")
+        self._run("pvg_render_bwd", C.byref(sc), ca, len(cams), frame.handle, dl, C.byref(g), _stream_ptr(stream))
         return grads
 
 
@@ -269,9 +284,10 @@ class _FrameLease:
     holds some 20 device buffers, and creating and freeing them was most of a
     small differentiable render.  An idle frame is only lent to the stream
     that used it last, behind whose work it is free: the stream itself, and
-    not one that was given a destroyed stream's handle.  A renderer keeps at
-    most ``KEEP`` idle frames and frees them with itself; a lease taken while
-    the stream is being captured is a frame of its own."""
+    not one that was given a destroyed stream's handle.  A renderer keeps the
+    ``KEEP`` idle frames used last, gives them up when device memory runs out
+    and frees them with itself; a lease taken while the stream is being
+    captured is a frame of its own."""
 
     KEEP = 4
 
@@ -282,15 +298,14 @@ class _FrameLease:
         self.own = torch.cuda.is_current_stream_capturing()
         if not self.own:
             self.key = _stream_key(self.stream)
-            for _ in range(len(renderer._frames)):
-                try:
-                    stream, frame = renderer._frames.pop()
-                except IndexError:  # another thread's
+            for entry in reversed(tuple(renderer._frames)):
+                if entry[1].stream_key == self.key:
+                    try:
+                        renderer._frames.remove(entry)
+                    except ValueError:  # another thread's
+                        continue
+                    self.frame = entry[1]
                     break
-                if frame.stream_key == self.key:
-                    self.frame = frame
-                    break
-                renderer._frames.insert(0, (stream, frame))
         if self.frame is None:
             self.frame = Frame()
 
@@ -305,12 +320,16 @@ class _FrameLease:
             return
         r = self.renderer
         handle = self.stream.cuda_stream
-        if (self.own or r.handle is None or (stream is not None and stream.cuda_stream != handle)
-                or len(r._frames) >= self.KEEP):
+        if self.own or r.handle is None or (stream is not None and stream.cuda_stream != handle):
             frame.close()
-        else:
-            frame.stream_key = self.key
-            r._frames.append((handle, frame))
+            return
+        frame.stream_key = self.key
+        r._frames.append((handle, frame))
+        while len(r._frames) > self.KEEP:
+            try:
+                r._frames.pop(0)[1].close()
+            except IndexError:  # another thread's
+                break
 
     def __del__(self):
         try:
@@ -399,9 +418,8 @@ def l1_loss(renderer, pred, target, dl=None, loss=None, scale=None, stream=None)
     if loss is None:
         loss = torch.empty(1, device=pred.device, dtype=torch.float32)
     s = 1.0 / max(n, 1) if scale is None else float(scale)
-    st = abi.lib().pvg_l1_loss(renderer.handle, pred.data_ptr(), target.data_ptr(), n, s, dl.data_ptr(),
-                              loss.data_ptr(), _stream_ptr(stream))
-    abi.check(st, "pvg_l1_loss")
+    renderer._run("pvg_l1_loss", pred.data_ptr(), target.data_ptr(), n, s, dl.data_ptr(), loss.data_ptr(),
+                  _stream_ptr(stream))
     return loss, dl
 
 
@@ -416,9 +434,8 @@ def rgb_loss(renderer, pred, target, lambda_r=0.2, dl=None, loss=None, stream=No
     if loss is None:
         loss = torch.empty(3, device=pred.device, dtype=torch.float32)
     C_, H, W = pred.shape
-    st = abi.lib().pvg_rgb_loss(renderer.handle, pred.data_ptr(), target.data_ptr(), int(C_), int(H), int(W),
-                               float(lambda_r), dl.data_ptr(), loss.data_ptr(), _stream_ptr(stream))
-    abi.check(st, "pvg_rgb_loss")
+    renderer._run("pvg_rgb_loss", pred.data_ptr(), target.data_ptr(), int(C_), int(H), int(W), float(lambda_r),
+                  dl.data_ptr(), loss.data_ptr(), _stream_ptr(stream))
     return loss, dl
 
 
@@ -467,9 +484,8 @@ def sort_pairs(renderer, keys, vals, begin_bit=0, end_bit=32, stream=None):
     ``vals`` by key bits [begin_bit, end_bit) (``pvg_sort_pairs``)."""
     if keys.shape != vals.shape or keys.dim() != 1 or not keys.is_contiguous() or not vals.is_contiguous():
         raise ValueError("keys and vals must be contiguous 1-D tensors of one length")
-    st = abi.lib().pvg_sort_pairs(renderer.handle, keys.data_ptr(), vals.data_ptr(), keys.numel(), int(begin_bit),
-                                  int(end_bit), _stream_ptr(stream))
-    abi.check(st, "pvg_sort_pairs")
+    renderer._run("pvg_sort_pairs", keys.data_ptr(), vals.data_ptr(), keys.numel(), int(begin_bit), int(end_bit),
+                  _stream_ptr(stream))
     return keys, vals
 
 
@@ -485,7 +501,6 @@ def render_multi(renderer, scenes, cams, outs=None, frame=None, stream=None):
     ca = abi.cameras(cams)
     imgs = (abi.Image * len(cams))()
     _fill_images(imgs, outs, 0)
-    st = abi.lib().pvg_render_fwd_multi(renderer.handle, sc, ca, len(cams), imgs,
-                                        frame.handle if frame is not None else None, _stream_ptr(stream))
-    abi.check(st, "pvg_render_fwd_multi")
+    renderer._run("pvg_render_fwd_multi", sc, ca, len(cams), imgs, frame.handle if frame is not None else None,
+                  _stream_ptr(stream))
     return outs

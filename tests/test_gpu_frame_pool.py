@@ -1,6 +1,7 @@
-"""The idle frames that a renderer keeps for render_differentiable are never
-lent to a stream that only has the handle of a destroyed one, outlive the
-stream that used them, and are never left to a captured backward pass.
+"""The idle frames that a renderer keeps for render_differentiable: bounded,
+the least recently used one dropped first, given up when memory runs out,
+never lent to a stream that only has the handle of a destroyed one, kept past
+the stream that used them, and never left to a captured backward pass.
 """
 import ctypes
 
@@ -40,6 +41,57 @@ def _step(st, r):
     g = _backward(*_forward(st, r))
     torch.cuda.synchronize()
     return g
+
+
+def test_the_least_recently_used_frame_is_dropped(scene):
+    r = R.Renderer()
+    streams = [torch.cuda.Stream() for _ in range(R._FrameLease.KEEP + 1)]
+    torch.cuda.synchronize()
+    for s in streams:
+        with torch.cuda.stream(s):
+            _step(scene, r)
+    kept = [f for _, f in r._frames]
+    assert len(kept) == R._FrameLease.KEEP
+    with torch.cuda.stream(streams[-1]):
+        assert R._FrameLease(r).frame is kept[-1]  # the last stream's own
+    with torch.cuda.stream(streams[0]):
+        assert R._FrameLease(r).frame not in kept  # dropped for it
+    r.close()
+    assert not r._frames
+
+
+def test_idle_frames_are_given_up_when_memory_runs_out(scene):
+    other = R.scene_to_device(synth.make_plain_scene(seed=3, n=20_000))
+    want = R.Renderer().forward(other, [CAM])[0]["rgb"].clone()
+    r = R.Renderer()
+    _step(scene, r)
+    assert len(r._frames) == 1
+    abi.lib().pvg_debug_fail_allocations(1)
+    out = r.forward(other, [CAM])[0]["rgb"]
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and not r._frames
+    # without idle frames the failure is the caller's
+    plain = R.Renderer()
+    abi.lib().pvg_debug_fail_allocations(1)
+    with pytest.raises(abi.PVGError) as e:
+        plain.forward(other, [CAM])
+    assert e.value.status == 2
+    # an idle frame gone, the backward pass that needs the memory runs too
+    abi.lib().pvg_debug_fail_allocations(0)
+    _step(scene, r)
+    p, out = _forward(scene, r)  # takes the idle frame
+    q, out2 = _forward(scene, r)
+    _backward(q, out2)           # leaves another
+    fr = R.Frame()
+    r.forward(other, [CAM], frame=fr)
+    abi.lib().pvg_debug_fail_allocations(1)
+    g = r.backward(other, [CAM], fr, [dict(rgb=torch.ones(3, 48, 64, device="cuda"))])
+    torch.cuda.synchronize()
+    assert torch.isfinite(g["mu"]).all() and not r._frames
+    _step(scene, r)
+    r.free_idle_frames()
+    assert not r._frames
+    _backward(p, out)
 
 
 def _external_stream():
