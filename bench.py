@@ -576,14 +576,13 @@ def run_ours(args):
         "data": "synthetic (seeded urban-shaped PVG scene, random-init parameters)",
         "config": {"workload": WORKLOAD, "gaussians": N_GAUSS, "width": W_PIX, "height": H_PIX,
                    "name": args.workload, "sh_degree": 3,
-                   "tile": "%dx%d, %d px/thread (%s)" % (best[0], best[1], best[2],
-                                                         "given" if table is None else "autotuned"),
+                   "tile": "%dx%d (%s)" % (best[0], best[1], "given" if table is None else "autotuned"),
                    "l2": "flushed before every step (256 MB write)",
                    "step": "one CUDA-graph replay of forward + L1 + backward (pair capacity %d = 2x the measured K, no host round trip)" % pair_capacity,
                    "parallelism": ("data parallel, gradients all-reduced" if dp else "replicas")
                    if world > 1 else "single GPU"},
         "fwd_bwd_step_ms": ms_step,
-        "autotune_ms": None if table is None else {"%dx%dx%d" % k: round(v, 4) for k, v in table.items()},
+        "autotune_ms": None if table is None else {"%dx%d" % k[:2]: round(v, 4) for k, v in table.items()},
         "render_fwd": {"ms": fwd_ms, "mpix_s": job_value(world, mpix, fwd_ms)},
         "stages_ms": {k: round(v, 4) for k, v in stage_ms.items()},
         "visible": M, "pairs": K, "evals": E, "blended_evals": B, "overflow": ov,
@@ -657,7 +656,7 @@ def training_leg(dev, steps, fp32):
     mpix = w * h / 1e6
     best = ts["best"]
     return {"workload": WORKLOADS["training"][4], "ms_per_step": ms, "mpix_s": mpix / (ms * 1e-3),
-            "tile": "%dx%d, %d px/thread (autotuned)" % best, "steps": steps, "gpu_launches_per_step": launches,
+            "tile": "%dx%d (autotuned)" % best[:2], "steps": steps, "gpu_launches_per_step": launches,
             "l2": "flushed before every step", "stages_ms": {k: round(v, 4) for k, v in stage_ms.items()},
             "visible": M, "pairs": K, "evals": E, "blended_evals": B, "overflow": ov,
             "roofline": dominant_roof(stage_ms, E, B, n, M, K, fp32),
@@ -711,7 +710,7 @@ def batched_leg(dev, steps, fp32):
     r1.close()
     f1.close()
     return {"workload": "batched: 64 views (22x1920x1280, 21x1242x375, 21x960x640), 3M Gaussians SH-3, "
-                        "fwd + L1 + bwd", "mpix_per_batch": mpix, "tile": "%dx%d, %d px/thread (autotuned)" % g.config,
+                        "fwd + L1 + bwd", "mpix_per_batch": mpix, "tile": "%dx%d (autotuned)" % g.config[:2],
             "pair_capacity": g.pair_capacity, "overflow": over, "visible": M, "pairs": K, "evals": E,
             "blended_evals": B,
             "graph": {"ms": ms_graph, "mpix_s": mpix / (ms_graph * 1e-3)},

@@ -204,13 +204,12 @@ typedef struct {
                              * capacities below; pairs beyond the capacity are
                              * dropped and pvg_frame_stats reports the
                              * overflow (the images are then incomplete) */
-    int32_t pixels_per_thread; /* compositing pixels per thread (1, 2 or 4; 0 = 1).
-                             * Supported (tile_w, tile_h, pixels_per_thread):
-                             * (16,16,1|2|4) (8,8,1|2) (16,8,1|2) (32,8,1)
-                             * (32,16,1|2|4) (32,32,4) (16,32,4).  Checked and kept
-                             * with the frame; the kernels choose their pixels
-                             * per lane by the frame's size.  Images do not
-                             * depend on the choice (bit-identical). */
+    int32_t pixels_per_thread; /* 1, 2 or 4 (0 = 1).  Supported (tile_w, tile_h,
+                             * pixels_per_thread): (16,16,1|2|4) (8,8,1|2)
+                             * (16,8,1|2) (32,8,1) (32,16,1|2|4) (32,32,4)
+                             * (16,32,4).  Checked, and without effect: the
+                             * kernels choose their pixels per lane by the
+                             * frame's size (images are bit-identical). */
     int64_t pair_capacity;  /* pairs per frame when sync_sizes = 0 */
     float dilation;         /* EWA low-pass h in px^2 (default 0.3) */
     float fov_clamp;        /* J clamp factor (default 1.3) */

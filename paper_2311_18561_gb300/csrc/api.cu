@@ -199,7 +199,7 @@ struct pvg_frame {
     int feat_mask = 0, n_feat = 0, n_sem = 0;  // extra channels of the forward
     bool one_scene = true;      // every view renders the same scene
     uint32_t n_items = 0, total_tiles = 0, total_pix = 0, pair_capacity = 0;
-    int tile_w = 0, tile_h = 0, px = 1;
+    int tile_w = 0, tile_h = 0;
     int64_t n = -1;
     int sh_degree = -1;
     float dilation = 0.f;
@@ -605,7 +605,6 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
     f->total_pix = pix;
     f->tile_w = x->cfg.tile_w;
     f->tile_h = x->cfg.tile_h;
-    f->px = x->cfg.pixels_per_thread ? x->cfg.pixels_per_thread : 1;
     f->n = views[0].n;
     f->sh_degree = views[0].sh_degree;
     f->dilation = x->cfg.dilation;
@@ -626,7 +625,6 @@ static pvg_status_t enqueue_forward(pvg_ctx_t *x, pvg_frame *f, std::vector<View
     p.sh_degree = views[0].sh_degree;
     p.tile_w = x->cfg.tile_w;
     p.tile_h = x->cfg.tile_h;
-    p.px = f->px;
     p.dilation = x->cfg.dilation;
     p.n_items = NV;
     p.total_tiles = tiles;
@@ -933,7 +931,6 @@ extern "C" pvg_status_t pvg_render_bwd(pvg_ctx_t *x, const pvg_scene_t *scene, c
     p.sh_degree = scene->sh_degree;
     p.tile_w = f->tile_w;
     p.tile_h = f->tile_h;
-    p.px = f->px;
     p.dilation = f->dilation;
     p.n_items = f->n_items;
     p.total_tiles = f->total_tiles;
@@ -1117,7 +1114,6 @@ extern "C" pvg_status_t pvg_frame_eval_count(pvg_ctx_t *x, pvg_frame_t *f, int64
     p.n_views = nv;
     p.tile_w = f->tile_w;
     p.tile_h = f->tile_h;
-    p.px = f->px;
     p.total_tiles = f->total_tiles;
     p.total_pix = f->total_pix;
     p.rec = ptr<float4>(f->rec);

@@ -82,7 +82,6 @@ struct Params {
     int32_t n_views;
     int32_t sh_degree;       // of the call's scene (kernels are specialised on it)
     int32_t tile_w, tile_h;
-    int32_t px;              // pixels per compositing thread of the configuration
     int32_t block_shift;     // log2 of the width of a warp's pixel block (compositing kernels)
     uint32_t blocks_per_tile;  // warps' pixel blocks in a tile
     float dilation;

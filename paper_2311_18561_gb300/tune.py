@@ -1,11 +1,13 @@
 """Autotuner for the compositing configuration.
 
-The compositor's tile shape and pixels per thread change only speed: every
-supported configuration produces bit-identical images (each pixel's
-arithmetic is the same expression; the tile binning is conservative for
-the alpha gate).  So the tuner may pick any of them by time alone: it
-renders the caller's workload (forward, optionally forward + backward) with
-every candidate, times each with CUDA events, and returns the fastest.
+The compositor's tile shape changes only speed: every supported shape
+produces bit-identical images (each pixel's arithmetic is the same
+expression; the tile binning is conservative for the alpha gate).  So the
+tuner may pick any of them by time alone: it renders the caller's workload
+(forward, optionally forward + backward) with every candidate, times each
+with CUDA events, and returns the fastest.  The pixels per lane are the
+library's own choice, by the frame's size; a configuration's third number
+is accepted and checked, and one candidate per shape is enough.
 Results are cached in a JSON file keyed by the workload's shape (Gaussian
 count, SH degree, image sizes, whether the backward is included).
 """
@@ -18,9 +20,8 @@ import torch
 
 from . import render as R
 
-# every (tile width, tile height, pixels per thread) the library supports
-CONFIGS = ((16, 16, 1), (16, 16, 2), (16, 16, 4), (8, 8, 1), (8, 8, 2), (16, 8, 1), (16, 8, 2), (32, 8, 1),
-           (32, 16, 1), (32, 16, 2), (32, 16, 4), (32, 32, 4), (16, 32, 4))
+# one supported (tile width, tile height, pixels per thread) of every tile shape
+CONFIGS = ((16, 16, 1), (8, 8, 1), (16, 8, 1), (32, 8, 1), (32, 16, 1), (32, 32, 4), (16, 32, 4))
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "pvg_gb300", "tune.json")
 
