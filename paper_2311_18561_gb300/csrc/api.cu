@@ -189,7 +189,7 @@ struct pvg_frame {
     DevBuf pair_vals;           // [K]
     DevBuf ranges;              // [tiles]
     DevBuf tile_order;          // [tiles] compositor launch order
-    DevBuf tile_walk;           // [tiles] largest last-blend position per tile (forward)
+    DevBuf tile_walk;           // [tiles] largest stop position per tile (forward)
     DevBuf tile_order_bwd;      // [tiles] adjoint launch order (by walk)
     DevBuf pix_T, pix_last;     // [pixels]
     DevBuf pix_neval;           // [pixels]
@@ -960,7 +960,7 @@ extern "C" pvg_status_t pvg_render_bwd(pvg_ctx_t *x, const pvg_scene_t *scene, c
     if (capturing) tm.on = false;
     tm.begin(PVG_STAGE_COMPOSITE_BWD, s);
     // g2d zeroed, and the adjoint's tiles ordered longest walk first (the
-    // forward recorded each tile's largest last-blend position)
+    // forward recorded each tile's largest stop position)
     launch_bwd_prep(p, ptr<uint32_t>(f->tile_walk), ptr<uint32_t>(f->tile_order_bwd), s);
     p.tile_order = ptr<uint32_t>(f->tile_order_bwd);
     if (feat_bwd && f->n_items) {

@@ -10,14 +10,12 @@
 // so one scalar per pixel carries what the colour, depth and opacity
 // suffix sums would.  The image-space gradient terms of an entry (moments of
 // dL/dpower; r g b; z) are summed over a lane's pixels, then over the warp
-// (flush_terms) and added to the Gaussian's row in global memory.  Alpha is the forward's expression (explicit roundings), so the
-// blend decisions are the forward's; the rest of this file may contract
-// a*b+c into fused multiply-adds.
+// (flush_terms) and added to the Gaussian's row in global memory.  Alpha is the
+// forward's expression (explicit roundings), so the blend decisions are the
+// forward's; the rest of this file may contract a*b+c into fused multiply-adds.
 #include "raster_bwd.cuh"
 
 namespace pvg {
-namespace {
-}  // namespace
 
 void launch_composite_bwd(const Params &p, cudaStream_t s) {
     if (p.total_tiles == 0) return;

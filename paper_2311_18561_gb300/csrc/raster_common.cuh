@@ -55,7 +55,9 @@ __device__ __forceinline__ BlockGeom block_geom(const Params &P) {
 // edge's own maximum clamped into it.  The level is widened by 1 % + 1e-4
 // against the rounding of the compositor's own evaluation, and needle
 // footprints ((a + c)^2 > 1e4 (ac - b^2), where that rounding may exceed it)
-// and non-finite entries always count as hits, so culling changes no image.
+// and conics that are not finite always count as hits; an entry whose position
+// or opacity is NaN may be culled, since its alpha test is false at every
+// pixel.  So culling changes no image.
 __device__ __forceinline__ bool block_hit(float u, float v, float ap, float bp, float cp, float ot, float x0,
                                           float x1, float y0, float y1) {
     const float hb = 0.5f * bp, tr = ap + cp;

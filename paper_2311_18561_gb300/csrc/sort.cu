@@ -894,7 +894,7 @@ void scan_emit_pairs(const Params &p, void *temp, cudaStream_t s) {
 // and the short ones fill in behind them.  Order within a bucket is left
 // to the atomics (each tile's result does not depend on when it runs).
 // walk (optional): order by the tiles' walk lengths instead (the adjoint:
-// each tile's largest last-blend position, which the forward recorded).
+// each tile's largest stop position, which the forward recorded).
 // One cluster of kOrderCtas CTAs (rank: this one's), which count their
 // shares of the tiles and read one another's counts; a warp adds once per
 // bucket it meets (with 55,000 tiles one CTA with an atomic per tile took 60

@@ -20,11 +20,13 @@
 // the gradient; the per-CTA sums of S and |x - y| go to a partial array
 // that one small kernel adds in a fixed order (the loss is deterministic).
 //
-// Bound by issue slots (the taps alone are 349 multiply-adds per pixel and
-// channel with the halos, 26 bytes of HBM), so every filter runs on packed
-// pairs: a row pass filters two rows at once, a column pass two columns, and
-// the values a row pass reads are stored as row pairs.  Each half rounds as
-// the scalar filter did.
+// The taps are 349 multiply-adds per pixel and channel with the halos (26
+// bytes of HBM).  Every filter runs on packed pairs: a row pass filters two
+// rows at once, a column pass two columns, and the values a row pass reads are
+// stored as row pairs (3x1280x1920: 190 us by scalars, 175 us).  Each half
+// rounds as the scalar filter did.  Nothing is full: 64 % of the shared-memory
+// wavefronts, 54 % of the issue slots and 47 % of the FMA pipe at 17 warps per
+// SM, which wait for one another's halos at the barriers between the passes.
 #include <cooperative_groups.h>
 
 #include <utility>
