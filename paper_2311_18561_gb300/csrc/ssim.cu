@@ -20,7 +20,7 @@
 // the gradient; the per-CTA sums of S and |x - y| go to a partial array
 // that one small kernel adds in a fixed order (the loss is deterministic).
 //
-// The taps are 349 multiply-adds per pixel and channel with the halos (26
+// The taps are 288 multiply-adds per pixel and channel with the halos (26
 // bytes of HBM).  Every filter runs on packed pairs: a row pass filters two
 // rows at once, a column pass two columns, and the values a row pass reads are
 // stored as row pairs (3x1280x1920: 190 us by scalars, 175 us).  Each half
