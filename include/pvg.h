@@ -228,9 +228,9 @@ void pvg_destroy(pvg_ctx_t *ctx);
 pvg_status_t pvg_set_config(pvg_ctx_t *ctx, const pvg_config_t *cfg);
 
 /* Saved state of one forward pass (depth-sorted visible Gaussians, their
- * projected records, per-tile lists, per-pixel final transmittance and last
- * blended position), needed by pvg_render_bwd.  A frame belongs to the
- * device that was current at creation. */
+ * projected records, per-tile lists, per-pixel final transmittance and stop
+ * position), needed by pvg_render_bwd.  A frame belongs to the device that was
+ * current at creation; destroying it waits for that device. */
 pvg_status_t pvg_frame_create(pvg_frame_t **frame);
 void pvg_frame_destroy(pvg_frame_t *frame);
 /* Counters of the last forward into `frame` (synchronises `frame`'s last

@@ -127,9 +127,9 @@ static Params with_shape(const Params &p, const WarpShape &w) {
 }
 
 // One pixel per lane: where four would not fill the SMs (warp_shape gives
-// two), and the lists are short.  With long lists the issue slots bound the
-// pass, the sooner the more blocks the SMs have; with hardly any entries the
-// blocks themselves do.  Measured with two / one pixel per lane, by items per
+// two), and the lists are short.  With long lists the instructions of all blocks
+// bound the pass, the sooner the more blocks the SMs have; with hardly any
+// entries the blocks themselves do.  Measured with two / one pixel per lane, by items per
 // block of 128 pixels, at 16 blocks per SM (641x479): 8: 23 / 20 us, 104: 95 /
 // 84, 416: 54 / 56; at 24 (1242x375): 16: 47 / 43, 69: 122 / 93, 137: 67 / 70,
 // 275: 71 / 80; at 46 (1000x900): 3: 25 / 29, 8: 43 / 41, 36: 86 / 78, 71: 78

@@ -18,8 +18,8 @@ constexpr int kFwdWarps4 = 16, kFwdWarps2 = 20;
 // Blocks of 128 pixels per SM from which a lane takes four pixels: below it
 // the longest walk bounds the pass and fewer pixels per lane shorten it
 // (four 640x480 views of 250k Gaussians, 9,100 blocks: 280 us with four, 186
-// us with two, 156 us with one); above it the issue slots do (1920x1280,
-// 19,200 blocks: 193, 243 and 313 us).
+// us with two, 156 us with one); above it the instructions of all blocks do
+// (1920x1280, 19,200 blocks: 193, 243 and 313 us).
 constexpr int kFwdWide = 64;
 // With one pixel per lane (four entries together: 156 us on those views,
 // eight 164 us).
