@@ -103,7 +103,7 @@ def _external_stream():
 
 
 def test_a_destroyed_streams_handle_does_not_lend_its_frames(scene):
-    """Whether a new stream gets a destroyed one's handle is the driver's
+    """Whether a new stream gets a destroyed one's handle is CUDA's own
     choice, so the idle frame is entered under a new stream's handle."""
     r = R.Renderer()
     handle, destroy = _external_stream()
